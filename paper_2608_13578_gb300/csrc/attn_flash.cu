@@ -571,6 +571,9 @@ __global__ void __launch_bounds__(128)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
+  O = after_wait(O);
+  dO = after_wait(dO);
+  lse = after_wait(lse);
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
@@ -767,6 +770,9 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
+  O = after_wait(O);
+  dO = after_wait(dO);
+  lse = after_wait(lse);
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
@@ -950,6 +956,8 @@ __global__ void __launch_bounds__(128)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
+  lse = after_wait(lse);
+  Drow = after_wait(Drow);
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, k0, b);
@@ -1139,6 +1147,8 @@ __global__ void __launch_bounds__(128, 3)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
+  lse = after_wait(lse);
+  Drow = after_wait(Drow);
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, k0, b);

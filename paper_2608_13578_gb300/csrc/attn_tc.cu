@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(128)
     tc::prefetch_tmap(&mO);
   }
   pdl_enter();
+  lse = after_wait(lse);
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(&bar[0], 5 * kT);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);

@@ -32,6 +32,16 @@ __device__ __forceinline__ void pdl_enter() {
   pdl_trigger();
   pdl_wait();
 }
+// A pointer to what an earlier kernel wrote, for use after pdl_wait().  The
+// compiler takes loads through a kernel's `const T* __restrict__` argument as
+// loads of constant memory and may move them above the wait, where they see the
+// previous contents; a pointer that comes out of this empty statement keeps its
+// loads below it (volatile statements stay in order).
+template <class T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
 
 // Host: while `on`, this thread's launches on `stream` carry `priority`
 // instead of the stream's own (the C-ABI calls raise their critical chain,

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(1024)
     decode_gemv_kernel(const float* __restrict__ A, int M, int K, const TW* __restrict__ W, int N,
                        float* __restrict__ out, int round_out) {
   pdl_enter();
+  A = after_wait(A);
   constexpr int KC = 256;  // K chunk staged in shared memory
   __shared__ float sA[R][KC];
   extern __shared__ float red[];  // [32 warps][R][33]
@@ -94,6 +95,9 @@ __global__ void __launch_bounds__(128)
     decode_attn_kernel(const float* __restrict__ qkv, T* __restrict__ Kc, T* __restrict__ Vc,
                        float* __restrict__ hhat, int D, int dh, int L, int j, float scale) {
   pdl_enter();
+  qkv = after_wait(qkv);
+  Kc = after_wait(Kc);
+  Vc = after_wait(Vc);
   __shared__ float q[128];
   __shared__ float p[kMaxL];
   __shared__ float red[2][4];
@@ -168,6 +172,14 @@ __global__ void __launch_bounds__(256)
                        float* __restrict__ Mr, T* __restrict__ y, int D, int j, int last,
                        int honly) {
   pdl_enter();
+  Hr = after_wait(Hr);
+  U = after_wait(U);
+  Cm = after_wait(Cm);
+  pm = after_wait(pm);
+  pden = after_wait(pden);
+  pnum = after_wait(pnum);
+  Nn = after_wait(Nn);
+  Zz = after_wait(Zz);
   __shared__ float red[8];
   const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* h = Hr + (long)b * D;
@@ -269,6 +281,7 @@ template <class T>
 __global__ void __launch_bounds__(256) decode_widen_kernel(const T* __restrict__ x, float* out,
                                                            long n) {
   pdl_enter();
+  x = after_wait(x);
   for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += (long)gridDim.x * 256)
     out[i] = to_f(x[i]);
 }

@@ -41,6 +41,8 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, con
                                                         const TI* __restrict__ B, long sbk,
                                                         long sbn, Epi epi, int kps) {
   pdl_enter();
+  A = after_wait(A);
+  B = after_wait(B);
   __shared__ float As[16][64 + 4];
   __shared__ float Bs[16][64 + 4];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -1360,7 +1362,7 @@ __global__ void reduce_splits_kernel(const __grid_constant__ RedSegs<TO> R) {
   int q = 0;
   while (q < R.n && i4 >= R.count[q]) i4 -= R.count[q++];
   if (q >= R.n) return;
-  const float* part = R.part[q];
+  const float* part = after_wait(R.part[q]);
   const long count = R.count[q];
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4

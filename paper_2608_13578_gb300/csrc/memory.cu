@@ -225,16 +225,19 @@ __device__ void gate_bwd_item(float* sm, const T* __restrict__ dY, const T* __re
   const T* gp = G + o0;
   T* dup = dU + o0;
   Raw8<T> rdy[RB], rgt[RB];
-  // dY is an input of the call, complete before the layer's first kernel
-  // started: its loads go out before the wait for the previous kernel (the
-  // caller's pdl_enter is here)
-#pragma unroll
-  for (int u = 0; u < RB; ++u)
-    if (cin && rg + 8 * u < n) ld_raw(dyp + u * step, rdy[u]);
+  // (the caller's pdl_enter is here.  dY waits too: this is the call's first
+  // kernel, and dY may be what a kernel still running writes, such as the dX
+  // of the layer above)
   pdl_enter();
+  dyp = after_wait(dyp);
+  gp = after_wait(gp);
+  Pm = after_wait(Pm);
 #pragma unroll
   for (int u = 0; u < RB; ++u)
-    if (cin && rg + 8 * u < n) ld_raw(gp + u * step, rgt[u]);
+    if (cin && rg + 8 * u < n) {
+      ld_raw(dyp + u * step, rdy[u]);
+      ld_raw(gp + u * step, rgt[u]);
+    }
   // meanwhile the memory row, one channel per thread, its K-split partials
   // summed in split order (C_0 = 0, C_i = P_{i-1})
   {
@@ -502,8 +505,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   const bf16* dYb = dY + rowbase * D;
   // dY goes straight to shared memory (cp.async: no registers held while it
   // is in flight), each thread's own pieces, read back by the same thread.
-  // dY is an input of the call, complete before the layer's first kernel
-  // started, so its copies go out before the wait for the previous kernel.
+  // dY was read by the call's first kernel, whose completion the memory
+  // gradient's stream (joined just before this launch) has waited for, so its
+  // copies go out before the wait for the previous kernel.
   extern __shared__ __align__(16) uint8_t ys_raw[];  // [8 RW rows][KC * 256] bf16
   bf16* ys = reinterpret_cast<bf16*>(ys_raw);
 #pragma unroll
@@ -517,6 +521,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
   cp_async_commit();
   pdl_enter();
+  Hb = after_wait(Hb);
+  dHb = after_wait(dHb);
+  alpha = after_wait(alpha);
+  Sb = after_wait(Sb);
+  dS = after_wait(dS);
   if (n <= 0) {  // a ragged last block's empty chunk: zero partials of dW_p
     for (int k = threadIdx.x; k < D; k += kThreads) dwp_part[prow * D + k] = 0.f;
     return;
@@ -623,6 +632,8 @@ __global__ void __launch_bounds__(kThreads)
                        long n_tok, float* __restrict__ alpha, float* __restrict__ S, int Tlen,
                        int D, int L, int Nb) {
   pdl_enter();
+  Hm = after_wait(Hm);
+  spart = after_wait(spart);
   extern __shared__ __align__(16) float sm[];
   const int i = blockIdx.x, b = blockIdx.y, z = blockIdx.z;
   const float Si = pool_block<T>(sm, Hm, spart, npart, n_tok, alpha, Tlen, D, L, i, b, z);
@@ -661,6 +672,7 @@ __global__ void __launch_bounds__(kPsThreads)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = x * kPsCh;
   pdl_enter();
+  S = after_wait(S);
   // the carry of the earlier windows, per channel this warp scans
   float cn[kPsCh / 8], cz[kPsCh / 8];
 #pragma unroll
@@ -895,6 +907,7 @@ __global__ void __launch_bounds__(kProjThreads)
     apre[q] = k < D ? decay[k] : 0.f;
   }
   pdl_enter();
+  S = after_wait(S);
   // the batch's summaries to shared memory in 16-byte pieces (all in flight
   // at once, no registers held)
   {
@@ -990,6 +1003,9 @@ __global__ void __launch_bounds__(kScanThreads)
                            const float* __restrict__ M, float* __restrict__ dS,
                            float* __restrict__ da_part, int Nb, int D) {
   pdl_enter();
+  dM = after_wait(dM);
+  Z = after_wait(Z);
+  M = after_wait(M);
   scan_bwd_item<PS>(dM, mstride, decay, Z, M, dS, da_part, Nb, D, blockIdx.x, blockIdx.y);
 }
 
@@ -1001,6 +1017,11 @@ __global__ void __launch_bounds__(kThreads, 2)
                        float* __restrict__ ds, float* __restrict__ dwp_part, int Tlen, int D,
                        int L, int Nb) {
   pdl_enter();
+  Hm = after_wait(Hm);
+  alpha = after_wait(alpha);
+  Sb = after_wait(Sb);
+  dS = after_wait(dS);
+  dH = after_wait(dH);
   __shared__ __align__(16) float sm[ROWS + 8 + 8 * 260];
   // a ragged last block has fewer chunks than the grid's x extent: its empty
   // chunks contribute zero partials to dW_p
@@ -1028,6 +1049,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     inject_kernel(const T* __restrict__ Hm, const T* __restrict__ G, const float* __restrict__ Pm,
                   long pstride, T* __restrict__ Y, int B, int Tlen, int D, int L, int Nb) {
   pdl_enter();
+  Hm = after_wait(Hm);
+  G = after_wait(G);
+  Pm = after_wait(Pm);
   constexpr int kInjRows = inj_rows(sizeof(T));
   const int runs = D / 8, groups = (L + kInjRows - 1) / kInjRows;
   const long total = (long)B * Nb * groups * runs;
@@ -1271,6 +1295,7 @@ template <class TO>
 __global__ void __launch_bounds__(256)
     reduce_rows_kernel(const float* __restrict__ in, int rows, int cols, TO* __restrict__ out) {
   pdl_enter();
+  in = after_wait(in);
   __shared__ float part[8][33];
   const int rg = threadIdx.x >> 5, cl = threadIdx.x & 31;
   const int c = blockIdx.x * 32 + cl;
