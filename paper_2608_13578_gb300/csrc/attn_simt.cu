@@ -1,192 +1,681 @@
-// Intra-block causal multi-head attention on CUDA cores (Sec. 3.3), forward
-// and backward.  Used for fp32 tensors (true fp32 arithmetic) and for bf16
-// shapes the tensor-core kernel does not cover.  One warp per query row
-// (forward, dQ) or key row (dK, dV); each lane owns keys (scores) or channels
-// (outputs).  Deterministic: every sum runs in a fixed order.
+// Intra-block causal multi-head attention on CUDA cores (Sec. 3.3): forward and
+// backward of fp32 tensors (true fp32 arithmetic throughout), the forward of
+// the bf16 shapes that attn_tc.cu and attn_flash.cu do not take, the backward
+// that allocates nothing, and every bf16 shape when the tensor-core kernels are
+// switched off.
+//
+// One CTA of 256 threads (16 x 16) per 64-token tile of one head.  For L <= 64 a
+// tile holds the 64 / L whole blocks that fit and is its own key tile; for
+// L > 64 it is up to 64 rows of one block and walks the block's tiles.  Tiles lie
+// in shared memory as fp32 rows padded by 4 (the 8 rows that a quarter-warp's
+// 16-byte loads touch fall in distinct banks).  A thread holds a 4 x 4 block of
+// scores (rows 4 ty .. +3, columns tx + 16 j): 64 multiply-adds for every eight
+// 16-byte loads.  In the products over keys or queries it holds four columns
+// (twice four for heads above 64) of one, two or four rows, so that all threads
+// have outputs at every head width, and skips what the causal mask hides from
+// its rows.  Bound: fp32 issue, shared-memory bandwidth close behind.  Before,
+// one warp per query row read every key row from L2; times before and now:
+// B8 T1024 D512 h8 L64 fp32 forward 516 and 59 us, backward 2002 and 120 us;
+// B4 T2048 D1024 h8 L128 bf16 forward 1997 and 172 us; B4 T1000 D768 h8 L48 bf16
+// forward 306 and 61 us.  Deterministic: every sum runs in a fixed order.
 #include <mutex>
 
+#include "attn_slow.cuh"
 #include "common.cuh"
 #include "internal.h"
 
 namespace bcmt {
 
 namespace {
-constexpr int kMaxL = 1024;   // longest block the SIMT kernels accept
+constexpr int kMaxL = 1024;   // longest block
 constexpr int kMaxDh = 128;   // widest head
-constexpr int kWarps = 4;
+constexpr int kTile = 64;
+constexpr int kThreads = 256;
+constexpr int kPld = kTile + 4;  // row stride of a score tile
+
+template <class E>
+struct SimtArgs {
+  AttnPtrs<E> x;
+  E *Out, *dQ, *dK, *dV;
+  long ld_d;
+  float *lse, *Drow;
+  int rows;  // L <= 64: rows per tile (whole blocks)
+  int tpb;   // L > 64: tiles per block
+  int vec;   // rows of every tensor are aligned to four elements
+};
+
+struct TileAt {
+  int t0, rows, kstart, j;
+};
+template <class E>
+__device__ __forceinline__ TileAt tile_at(const SimtArgs<E>& a, int x) {
+  TileAt t;
+  if (a.x.L <= kTile) {
+    t.t0 = t.kstart = x * a.rows;
+    t.j = 0;
+    t.rows = min(a.rows, a.x.T - t.t0);
+  } else {
+    const int i = x / a.tpb;
+    t.j = x - i * a.tpb;
+    t.kstart = i * a.x.L;
+    t.t0 = t.kstart + t.j * kTile;
+    t.rows = min(min(kTile, a.x.L - t.j * kTile), a.x.T - t.t0);
+  }
+  return t;
+}
+
+// Rows [0, rows) x dh columns of a head into a tile, the other rows zero; a
+// thread's loads of four rows go out together.
+template <class E>
+__device__ __forceinline__ void fill(float* dst, int ldh, const E* src, long ld, int rows, int dh,
+                                     bool vec) {
+  const int r0 = threadIdx.x >> 4;
+  for (int c = (threadIdx.x & 15) * 4; c < dh; c += 64) {
+    float v[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + 16 * u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[u][e] = 0.f;
+      if (r < rows) {
+        const E* p = src + (long)r * ld + c;
+        if (vec) {
+          load4(p, v[u]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[u][e] = to_f(p[e]);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      *reinterpret_cast<float4*>(dst + (r0 + 16 * u) * ldh + c) =
+          make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+  }
+}
+template <class E>
+__device__ __forceinline__ void put4(E* p, const float* v, bool vec) {
+  if (vec) {
+    store4(p, v);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) p[e] = from_f<E>(v[e]);
+  }
+}
+
+// s[i][j] = A[4 ty + i] . B[tx + 16 j] over dh columns, each a single chain in
+// column order.
+__device__ __forceinline__ void scores_in_order(const float* A, const float* B, int ldh, int dh,
+                                                float (*s)[4]) {
+  const float* pa = A + 4 * (threadIdx.x >> 4) * ldh;
+  const float* pb = B + (threadIdx.x & 15) * ldh;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+#pragma unroll 2
+  for (int k = 0; k < dh; k += 4) {
+    float4 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(pa + i * ldh + k);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        s[i][j] = fmaf(x[i].x, y[j].x, s[i][j]);
+        s[i][j] = fmaf(x[i].y, y[j].y, s[i][j]);
+        s[i][j] = fmaf(x[i].z, y[j].z, s[i][j]);
+        s[i][j] = fmaf(x[i].w, y[j].w, s[i][j]);
+      }
+  }
+}
+
+// The same with two chains per score (even and odd columns), as packed pairs.
+__device__ __forceinline__ void scores(const float* A, const float* B, int ldh, int dh,
+                                       float (*s)[4]) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  float2 acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  const float* pa = A + (4 * ty) * ldh;
+  const float* pb = B + tx * ldh;
+#pragma unroll 2
+  for (int k = 0; k < dh; k += 4) {
+    float4 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(pa + i * ldh + k);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].y), make_float2(y[j].x, y[j].y), acc[i][j]);
+        acc[i][j] = __ffma2_rn(make_float2(x[i].z, x[i].w), make_float2(y[j].z, y[j].w), acc[i][j]);
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s[i][j] = acc[i][j].x + acc[i][j].y;
+}
+
+// The thread's outputs: column group threadIdx.x % C4 (four columns, CB times 64
+// apart) of RT consecutive rows; 64 rows x C4 groups over 256 threads.
+template <int C4, int CB>
+struct Cols {
+  static constexpr int RT = C4 / 4;
+  __device__ __forceinline__ static int col() { return (threadIdx.x & (C4 - 1)) * 4; }
+  __device__ __forceinline__ static int row() { return (threadIdx.x / C4) * RT; }
+};
+
+// acc[i] += sum over keys j in [lo, hi), in order, of P[row + i][j] B[j - b0].
+template <int C4, int CB>
+__device__ __forceinline__ void rows_times(const float* P, int ldp, const float* B, int ldh, int dh,
+                                           int lo, int hi, int b0, float (*acc)[CB][4]) {
+  using C = Cols<C4, CB>;
+  const float* p = P + C::row() * ldp;
+  const int c = C::col();
+  if (c >= dh) return;
+#pragma unroll 4
+  for (int j = lo; j < hi; ++j) {
+    float w[C::RT];
+#pragma unroll
+    for (int i = 0; i < C::RT; ++i) w[i] = p[i * ldp + j];
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+      if (m == 0 || c + 64 * m < dh) {
+        const float4 v = *reinterpret_cast<const float4*>(B + (j - b0) * ldh + c + 64 * m);
+#pragma unroll
+        for (int i = 0; i < C::RT; ++i) {
+          acc[i][m][0] = fmaf(w[i], v.x, acc[i][m][0]);
+          acc[i][m][1] = fmaf(w[i], v.y, acc[i][m][1]);
+          acc[i][m][2] = fmaf(w[i], v.z, acc[i][m][2]);
+          acc[i][m][3] = fmaf(w[i], v.w, acc[i][m][3]);
+        }
+      }
+  }
+}
+// acc[i] += sum over queries r in [lo, hi) of P[r][row + i] B[r].
+template <int C4, int CB>
+__device__ __forceinline__ void cols_times(const float* P, const float* B, int ldh, int dh, int lo,
+                                           int hi, float (*acc)[CB][4]) {
+  using C = Cols<C4, CB>;
+  const float* p = P + C::row();
+  const int c = C::col();
+  if (c >= dh) return;
+#pragma unroll 4
+  for (int r = lo; r < hi; ++r) {
+    float w[C::RT];
+    if (C::RT == 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + r * kPld);
+      w[0] = x.x; w[C::RT > 1 ? 1 : 0] = x.y; w[C::RT > 2 ? 2 : 0] = x.z; w[C::RT > 3 ? 3 : 0] = x.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < C::RT; ++i) w[i] = p[r * kPld + i];
+    }
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+      if (m == 0 || c + 64 * m < dh) {
+        const float4 v = *reinterpret_cast<const float4*>(B + r * ldh + c + 64 * m);
+#pragma unroll
+        for (int i = 0; i < C::RT; ++i) {
+          acc[i][m][0] = fmaf(w[i], v.x, acc[i][m][0]);
+          acc[i][m][1] = fmaf(w[i], v.y, acc[i][m][1]);
+          acc[i][m][2] = fmaf(w[i], v.z, acc[i][m][2]);
+          acc[i][m][3] = fmaf(w[i], v.w, acc[i][m][3]);
+        }
+      }
+  }
+}
+template <int RT, int CB>
+__device__ __forceinline__ void zero(float (*acc)[CB][4]) {
+#pragma unroll
+  for (int i = 0; i < RT; ++i)
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][m][e] = 0.f;
+}
+__device__ __forceinline__ bool finite4(const float* v) {
+  return is_finite(v[0]) && is_finite(v[1]) && is_finite(v[2]) && is_finite(v[3]);
+}
+// sum over the 16 threads of a row group
+__device__ __forceinline__ float sum16(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ float max16(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+// First row of the block that row r of a tile belongs to (0 for L > 64: the
+// tile's whole walk is one block).
+__device__ __forceinline__ int block_row(int r, int L) { return L <= kTile ? (r / L) * L : 0; }
+__device__ __forceinline__ int block_end(int r, int L) {
+  return L <= kTile ? min((r / L) * L + L, kTile) : kTile;
+}
 }  // namespace
 
 // O[t] = sum_j softmax_j(q_t . k_j * scale) v_j over keys j in [blockstart(t), t].
-template <class T>
-__global__ void __launch_bounds__(kWarps * 32)
-    attn_fwd_simt_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
-                         long ld, T* __restrict__ O, long ld_o, float* __restrict__ lse, int Tlen,
-                         int H, int dh, int L, float scale) {
+//
+// The arithmetic and its order are those of one query at a time -- a score is
+// one chain of fused multiply-adds over the columns, the largest score of the
+// whole row is subtracted before any exponential, the sum runs in 32 interleaved
+// partials joined by a butterfly, the output is one chain over the keys -- so
+// the result does not depend on the tiling.  (A bf16 layer rounds O, H and the
+// gate to bf16 in turn: a last-bit difference here would move every later
+// rounding, the fp32 decay gradient among the results.)  Hence two phases: all
+// of the row's scores, kept in shared memory for up to kKeep key tiles (beyond
+// that they are formed twice), then exponentials, sum and output.
+constexpr int kKeep = 4;
+template <class E, int C4, int CB>
+__global__ void __launch_bounds__(kThreads, 2)
+    attn_fwd_simt_kernel(const __grid_constant__ SimtArgs<E> a, int ldp) {
   pdl_enter();
-  __shared__ float qs[kWarps][kMaxDh];
-  __shared__ float ps[kWarps][kMaxL];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kWarps + warp, h = blockIdx.y, b = blockIdx.z;
-  if (t >= Tlen) return;
-  const int bs = (t / L) * L, nk = t - bs + 1;
-  const long rowq = (long)b * Tlen + t;
+  using C = Cols<C4, CB>;
+  extern __shared__ __align__(16) float sm[];
+  const int dh = a.x.dh, ldh = dh + 4;
+  float *Qs = sm, *Ks = Qs + kTile * ldh, *Vs = Ks + kTile * ldh, *Ps = Vs + kTile * ldh,
+        *inv = Ps + kTile * ldp;  // [64]
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int h = blockIdx.y, b = blockIdx.z;
+  const TileAt tt = tile_at(a, blockIdx.x);
+  if (tt.rows <= 0) return;
+  const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
-  for (int c = lane; c < dh; c += 32) qs[warp][c] = to_f(Q[rowq * ld + c0 + c]);
-  __syncwarp();
-  float mx = -INFINITY;
-  for (int j = lane; j < nk; j += 32) {
-    const T* kr = K + ((long)b * Tlen + bs + j) * ld + c0;
-    float d = 0.f;
-    for (int c = 0; c < dh; ++c) d = fmaf(qs[warp][c], to_f(kr[c]), d);
-    d *= scale;
-    ps[warp][j] = d;
-    mx = fmaxf(mx, d);
+  const bool keep = ldp > kPld || tt.j == 0;
+  auto keys = [&](int kt) { return kt == tt.j ? tt.rows : kTile; };
+  auto load_tile = [&](float* dst, const E* src, int kt) {
+    fill(dst, ldh, src + (row0 + tt.kstart + kt * kTile) * a.x.ld + c0, a.x.ld, keys(kt), dh, a.vec);
+  };
+  // the thread's scaled scores of key tile kt (hidden keys -inf)
+  auto tile_scores = [&](int kt, float (*s)[4]) {
+    scores_in_order(Qs, Ks, ldh, dh, s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = 4 * ty + i, rbs = block_row(r, a.x.L);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int k = tx + 16 * j;
+        s[i][j] = (kt < tt.j || (k >= rbs && k <= r)) ? __fmul_rn(s[i][j], a.x.scale) : -INFINITY;
+      }
+    }
+  };
+  fill(Qs, ldh, a.x.Q + (row0 + tt.t0) * a.x.ld + c0, a.x.ld, tt.rows, dh, a.vec);
+  load_tile(Vs, a.x.V, 0);
+  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  for (int kt = 0; kt <= tt.j; ++kt) {
+    if (kt > 0) __syncthreads();
+    load_tile(Ks, a.x.K, kt);
+    __syncthreads();
+    float s[4][4];
+    tile_scores(kt, s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        mx[i] = fmaxf(mx[i], s[i][j]);
+        if (keep) Ps[(4 * ty + i) * ldp + kt * kTile + tx + 16 * j] = s[i][j];
+      }
   }
-  mx = warp_max(mx);
-  float sum = 0.f;
-  for (int j = lane; j < nk; j += 32) {
-    const float e = expf(ps[warp][j] - mx);
-    ps[warp][j] = e;
-    sum += e;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mx[i] = max16(mx[i]);
+
+  // exponentials of key tile kt into columns p0 .. of Ps
+  auto exps = [&](int kt, int p0) {
+    float s[4][4];
+    if (!keep) tile_scores(kt, s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float* p = Ps + (4 * ty + i) * ldp + p0 + tx + 16 * j;
+        *p = expf((keep ? *p : s[i][j]) - mx[i]);
+      }
+  };
+  if (keep)
+    for (int kt = 0; kt <= tt.j; ++kt) exps(kt, kt * kTile);
+  float acc[C::RT][CB][4], part[8];
+  zero<C::RT, CB>(acc);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) part[u] = 0.f;
+  const int warp = tid >> 5, lane = tid & 31;
+  for (int kt = 0; kt <= tt.j; ++kt) {
+    const int p0 = keep ? kt * kTile : 0;
+    __syncthreads();  // keep: the probabilities are written; else the last tile is used up
+    if (!keep) {
+      load_tile(Ks, a.x.K, kt);
+      load_tile(Vs, a.x.V, kt);
+      __syncthreads();
+      exps(kt, 0);
+      __syncthreads();
+    } else if (kt > 0) {
+      load_tile(Vs, a.x.V, kt);
+      __syncthreads();
+    }
+    // partial sums, warp w: rows 8w .. 8w+7, lane = key index in the block mod 32
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int r = 8 * warp + u, rbs = block_row(r, a.x.L);
+      const int n = kt < tt.j ? kTile : r + 1 - rbs;  // visible keys of this tile
+      for (int j = lane; j < n; j += 32) part[u] += Ps[r * ldp + p0 + rbs + j];
+    }
+    rows_times<C4, CB>(Ps, ldp, Vs, ldh, dh, p0 + (kt < tt.j ? 0 : block_row(C::row(), a.x.L)),
+                       p0 + (kt < tt.j ? kTile : min(C::row() + C::RT, tt.rows)), p0, acc);
   }
-  sum = warp_sum(sum);
-  __syncwarp();
-  const float inv = 1.0f / sum;
-  for (int c = lane; c < dh; c += 32) {
-    float acc = 0.f;
-    for (int j = 0; j < nk; ++j)
-      acc = fmaf(ps[warp][j], to_f(V[((long)b * Tlen + bs + j) * ld + c0 + c]), acc);
-    O[rowq * ld_o + c0 + c] = from_f<T>(acc * inv);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    part[u] = warp_sum(part[u]);
+    if (lane == u) inv[8 * warp + u] = part[u];
   }
-  if (lane == 0) lse[((long)b * H + h) * Tlen + t] = mx + logf(sum);
+  __syncthreads();
+  if (tx < 4 && 4 * ty + tx < tt.rows) {
+    const int r = 4 * ty + tx;
+    const float m = tx == 0 ? mx[0] : tx == 1 ? mx[1] : tx == 2 ? mx[2] : mx[3];
+    a.lse[((long)b * a.x.H + h) * a.x.T + tt.t0 + r] = m + logf(inv[r]);
+  }
+  const int c = C::col();
+#pragma unroll
+  for (int i = 0; i < C::RT; ++i) {
+    const int r = C::row() + i, t = tt.t0 + r;
+    if (r >= tt.rows) break;
+    const float in = 1.0f / inv[r];
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+      if (c + 64 * m < dh) {
+        float* v = acc[i][m];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] *= in;
+        if (!finite4(v)) slow_o<4>(a.x, b, h, t, c + 64 * m, v);
+        put4(a.Out + (row0 + t) * a.x.ld_o + c0 + c + 64 * m, v, true);
+      }
+  }
 }
 
-// Per query t: Drow_t = dO_t . O_t, and
-// dQ_t = scale * sum_j P_tj (dO_t . v_j - Drow_t) k_j.
-template <class T>
-__global__ void __launch_bounds__(kWarps * 32)
-    attn_bwd_q_simt_kernel(const T* __restrict__ Q, const T* __restrict__ K,
-                           const T* __restrict__ V, long ld, const T* __restrict__ O,
-                           const T* __restrict__ dO, long ld_o, const float* __restrict__ lse,
-                           float* __restrict__ Drow, T* __restrict__ dQ, long ld_d, int Tlen, int H,
-                           int dh, int L, float scale) {
+namespace {
+// Drow of the thread's four rows, from the tensors: the 16 threads of a row
+// group share a row's columns.
+template <class E>
+__device__ __forceinline__ void drow4(const SimtArgs<E>& a, const TileAt& tt, int b, int h,
+                                      float* d) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = 4 * ty + i;
+    float s = 0.f;
+    if (r < tt.rows) {
+      const long o = ((long)b * a.x.T + tt.t0 + r) * a.x.ld_o + h * a.x.dh;
+      for (int c = 4 * tx; c < a.x.dh; c += 64) {
+        float u[4], v[4];
+        load4(a.x.dO + o + c, u);
+        load4(a.x.O + o + c, v);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s = fmaf(u[e], v[e], s);
+      }
+    }
+    d[i] = sum16(s);
+  }
+}
+// P and dS = P (dP - Drow) scale of the thread's 4 x 4 block, rows past `rows`
+// and hidden keys 0.
+template <class E>
+__device__ __forceinline__ void p_ds(const SimtArgs<E>& a, const float* Qs, const float* Ks,
+                                     const float* Gs, const float* Vs, int ldh, bool diag, int rows,
+                                     const float* lse, const float* drow, float (*p)[4],
+                                     float (*ds)[4]) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  scores(Qs, Ks, ldh, a.x.dh, p);
+  scores(Gs, Vs, ldh, a.x.dh, ds);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = 4 * ty + i, rbs = block_row(r, a.x.L);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = tx + 16 * j;
+      const bool vis = r < rows && (!diag || (k >= rbs && k <= r));
+      p[i][j] = vis ? expf(p[i][j] * a.x.scale - lse[i]) : 0.f;
+      ds[i][j] = vis ? p[i][j] * (ds[i][j] - drow[i]) * a.x.scale : 0.f;
+    }
+  }
+}
+__device__ __forceinline__ void put_tile(float* P, const float (*v)[4]) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) P[(4 * ty + i) * kPld + tx + 16 * j] = v[i][j];
+}
+template <class E>
+__device__ __forceinline__ void rows_lse(const SimtArgs<E>& a, int b, int h, int t0, int rows,
+                                         const float* src, float* v) {
+  const int ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    v[i] = 4 * ty + i < rows ? src[((long)b * a.x.H + h) * a.x.T + t0 + 4 * ty + i] : 0.f;
+}
+template <class E, int C4, int CB>
+__device__ __forceinline__ void store_dq(const SimtArgs<E>& a, const TileAt& tt, int b, int h,
+                                         float (*acc)[CB][4]) {
+  using C = Cols<C4, CB>;
+  const int c = C::col();
+#pragma unroll
+  for (int i = 0; i < C::RT; ++i) {
+    const int r = C::row() + i, t = tt.t0 + r;
+    if (r >= tt.rows) break;
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+      if (c + 64 * m < a.x.dh) {
+        if (!finite4(acc[i][m])) slow_dq<4>(a.x, b, h, t, c + 64 * m, acc[i][m]);
+        put4(a.dQ + ((long)b * a.x.T + t) * a.ld_d + h * a.x.dh + c + 64 * m, acc[i][m], a.vec);
+      }
+  }
+}
+}  // namespace
+
+// L > 64, per query tile: Drow_t = dO_t . O_t, and
+// dQ_t = scale * sum_j P_tj (dO_t . v_j - Drow_t) k_j over the block's key tiles.
+template <class E, int C4, int CB>
+__global__ void __launch_bounds__(kThreads)
+    attn_bwd_q_simt_kernel(const __grid_constant__ SimtArgs<E> a) {
   pdl_enter();
-  __shared__ float qs[kWarps][kMaxDh];
-  __shared__ float gs[kWarps][kMaxDh];
-  __shared__ float ds[kWarps][kMaxL];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kWarps + warp, h = blockIdx.y, b = blockIdx.z;
-  if (t >= Tlen) return;
-  const int bs = (t / L) * L, nk = t - bs + 1;
-  const long rowq = (long)b * Tlen + t;
+  extern __shared__ __align__(16) float sm[];
+  const int dh = a.x.dh, ldh = dh + 4;
+  float *Qs = sm, *Gs = Qs + kTile * ldh, *Ks = Gs + kTile * ldh, *Vs = Ks + kTile * ldh,
+        *Ss = Vs + kTile * ldh;
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  const int h = blockIdx.y, b = blockIdx.z;
+  const TileAt tt = tile_at(a, blockIdx.x);
+  if (tt.rows <= 0) return;
+  const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
-  float dd = 0.f;
-  for (int c = lane; c < dh; c += 32) {
-    qs[warp][c] = to_f(Q[rowq * ld + c0 + c]);
-    const float g = to_f(dO[rowq * ld_o + c0 + c]);
-    gs[warp][c] = g;
-    dd = fmaf(g, to_f(O[rowq * ld_o + c0 + c]), dd);
+  fill(Qs, ldh, a.x.Q + (row0 + tt.t0) * a.x.ld + c0, a.x.ld, tt.rows, dh, a.vec);
+  fill(Gs, ldh, a.x.dO + (row0 + tt.t0) * a.x.ld_o + c0, a.x.ld_o, tt.rows, dh, true);
+  using C = Cols<C4, CB>;
+  float drow[4], lse[4], acc[C::RT][CB][4];
+  drow4(a, tt, b, h, drow);
+  rows_lse(a, b, h, tt.t0, tt.rows, a.lse, lse);
+  if (tx == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (4 * ty + i < tt.rows)
+        a.Drow[((long)b * a.x.H + h) * a.x.T + tt.t0 + 4 * ty + i] = drow[i];
   }
-  dd = warp_sum(dd);
-  __syncwarp();
-  const float lt = lse[((long)b * H + h) * Tlen + t];
-  for (int j = lane; j < nk; j += 32) {
-    const long rk = ((long)b * Tlen + bs + j) * ld + c0;
-    float s = 0.f, dp = 0.f;
-    for (int c = 0; c < dh; ++c) {
-      s = fmaf(qs[warp][c], to_f(K[rk + c]), s);
-      dp = fmaf(gs[warp][c], to_f(V[rk + c]), dp);
-    }
-    const float p = expf(s * scale - lt);
-    ds[warp][j] = p * (dp - dd);
+  zero<C::RT, CB>(acc);
+  for (int kt = 0; kt <= tt.j; ++kt) {
+    const bool diag = kt == tt.j;
+    const int k0 = tt.kstart + kt * kTile, nk = diag ? tt.rows : kTile;
+    if (kt > 0) __syncthreads();
+    fill(Ks, ldh, a.x.K + (row0 + k0) * a.x.ld + c0, a.x.ld, nk, dh, a.vec);
+    fill(Vs, ldh, a.x.V + (row0 + k0) * a.x.ld + c0, a.x.ld, nk, dh, a.vec);
+    __syncthreads();
+    float p[4][4], ds[4][4];
+    p_ds(a, Qs, Ks, Gs, Vs, ldh, diag, tt.rows, lse, drow, p, ds);
+    put_tile(Ss, ds);
+    __syncthreads();
+    rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, 0, diag ? min(C::row() + C::RT, nk) : kTile, 0, acc);
   }
-  __syncwarp();
-  for (int c = lane; c < dh; c += 32) {
-    float acc = 0.f;
-    for (int j = 0; j < nk; ++j) acc = fmaf(ds[warp][j], to_f(K[((long)b * Tlen + bs + j) * ld + c0 + c]), acc);
-    dQ[rowq * ld_d + c0 + c] = from_f<T>(acc * scale);
-  }
-  if (lane == 0) Drow[((long)b * H + h) * Tlen + t] = dd;
+  store_dq<E, C4, CB>(a, tt, b, h, acc);
 }
 
-// Per key j: dV_j = sum_t P_tj dO_t, dK_j = scale * sum_t P_tj (dO_t . v_j - Drow_t) q_t
-// over queries t in [j, blockend(j)).
-template <class T>
-__global__ void __launch_bounds__(kWarps * 32)
-    attn_bwd_kv_simt_kernel(const T* __restrict__ Q, const T* __restrict__ K,
-                            const T* __restrict__ V, long ld, const T* __restrict__ dO, long ld_o,
-                            const float* __restrict__ lse, const float* __restrict__ Drow,
-                            T* __restrict__ dK, T* __restrict__ dV, long ld_d, int Tlen, int H,
-                            int dh, int L, float scale) {
+// Per key tile: dV_j = sum_t P_tj dO_t, dK_j = scale * sum_t P_tj (dO_t . v_j - Drow_t) q_t
+// over queries t in [j, blockend(j)), tile by tile.  FUSED (L <= 64, where the
+// tile is its own and only query tile): Drow is formed here and dQ joins, one
+// pass instead of two.
+template <class E, int C4, int CB, bool FUSED>
+__global__ void __launch_bounds__(kThreads)
+    attn_bwd_kv_simt_kernel(const __grid_constant__ SimtArgs<E> a) {
   pdl_enter();
-  __shared__ float ks[kWarps][kMaxDh];
-  __shared__ float vs[kWarps][kMaxDh];
-  __shared__ float ps[kWarps][kMaxL];
-  __shared__ float ds[kWarps][kMaxL];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = blockIdx.x * kWarps + warp, h = blockIdx.y, b = blockIdx.z;
-  if (j >= Tlen) return;
-  const int be = min((j / L) * L + L, Tlen), nq = be - j;
-  const long rowk = (long)b * Tlen + j;
+  extern __shared__ __align__(16) float sm[];
+  const int dh = a.x.dh, ldh = dh + 4;
+  float *Ks = sm, *Vs = Ks + kTile * ldh, *Qs = Vs + kTile * ldh, *Gs = Qs + kTile * ldh,
+        *Ps = Gs + kTile * ldh, *Ss = Ps + kTile * kPld;
+  const int h = blockIdx.y, b = blockIdx.z;
+  const TileAt tt = tile_at(a, blockIdx.x);
+  if (tt.rows <= 0) return;
+  const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
-  for (int c = lane; c < dh; c += 32) {
-    ks[warp][c] = to_f(K[rowk * ld + c0 + c]);
-    vs[warp][c] = to_f(V[rowk * ld + c0 + c]);
-  }
-  __syncwarp();
-  const long lb = ((long)b * H + h) * Tlen;
-  for (int u = lane; u < nq; u += 32) {
-    const int t = j + u;
-    const long rq = ((long)b * Tlen + t);
-    float s = 0.f, dp = 0.f;
-    for (int c = 0; c < dh; ++c) {
-      s = fmaf(to_f(Q[rq * ld + c0 + c]), ks[warp][c], s);
-      dp = fmaf(to_f(dO[rq * ld_o + c0 + c]), vs[warp][c], dp);
+  fill(Ks, ldh, a.x.K + (row0 + tt.t0) * a.x.ld + c0, a.x.ld, tt.rows, dh, a.vec);
+  fill(Vs, ldh, a.x.V + (row0 + tt.t0) * a.x.ld + c0, a.x.ld, tt.rows, dh, a.vec);
+  using C = Cols<C4, CB>;
+  float dk[C::RT][CB][4], dv[C::RT][CB][4];
+  zero<C::RT, CB>(dk);
+  zero<C::RT, CB>(dv);
+  const int jend = FUSED ? 1 : (min(a.x.L, a.x.T - tt.kstart) + kTile - 1) / kTile;
+  for (int i = tt.j; i < jend; ++i) {
+    const bool diag = i == tt.j;
+    const int t0 = FUSED ? tt.t0 : tt.kstart + i * kTile;
+    const int rows = FUSED ? tt.rows : min(min(kTile, a.x.L - i * kTile), a.x.T - t0);
+    if (!diag) __syncthreads();
+    fill(Qs, ldh, a.x.Q + (row0 + t0) * a.x.ld + c0, a.x.ld, rows, dh, a.vec);
+    fill(Gs, ldh, a.x.dO + (row0 + t0) * a.x.ld_o + c0, a.x.ld_o, rows, dh, true);
+    float drow[4], lse[4];
+    if (FUSED)
+      drow4(a, tt, b, h, drow);
+    else
+      rows_lse(a, b, h, t0, rows, a.Drow, drow);
+    rows_lse(a, b, h, t0, rows, a.lse, lse);
+    __syncthreads();
+    {
+      float p[4][4], ds[4][4];
+      p_ds(a, Qs, Ks, Gs, Vs, ldh, diag, rows, lse, drow, p, ds);
+      put_tile(Ps, p);
+      put_tile(Ss, ds);
     }
-    const float p = expf(s * scale - lse[lb + t]);
-    ps[warp][u] = p;
-    ds[warp][u] = p * (dp - Drow[lb + t]);
+    __syncthreads();
+    // the queries that see any of the thread's keys
+    const int lo = diag ? C::row() : 0;
+    const int hi = min(rows, diag ? block_end(C::row() + C::RT - 1, a.x.L) : kTile);
+    cols_times<C4, CB>(Ps, Gs, ldh, dh, lo, hi, dv);
+    cols_times<C4, CB>(Ss, Qs, ldh, dh, lo, hi, dk);
   }
-  __syncwarp();
-  for (int c = lane; c < dh; c += 32) {
-    float av = 0.f, ak = 0.f;
-    for (int u = 0; u < nq; ++u) {
-      const long rq = (long)b * Tlen + j + u;
-      av = fmaf(ps[warp][u], to_f(dO[rq * ld_o + c0 + c]), av);
-      ak = fmaf(ds[warp][u], to_f(Q[rq * ld + c0 + c]), ak);
-    }
-    dV[rowk * ld_d + c0 + c] = from_f<T>(av);
-    dK[rowk * ld_d + c0 + c] = from_f<T>(ak * scale);
+  const int c = C::col();
+#pragma unroll
+  for (int i = 0; i < C::RT; ++i) {
+    const int r = C::row() + i, t = tt.t0 + r;
+    if (r >= tt.rows) break;
+#pragma unroll
+    for (int m = 0; m < CB; ++m)
+      if (c + 64 * m < dh) {
+        if (!(finite4(dk[i][m]) && finite4(dv[i][m])))
+          slow_dkv<4>(a.x, b, h, t, c + 64 * m, dk[i][m], dv[i][m]);
+        const long o = (row0 + t) * a.ld_d + c0 + c + 64 * m;
+        put4(a.dV + o, dv[i][m], a.vec);
+        put4(a.dK + o, dk[i][m], a.vec);
+      }
+  }
+  if (FUSED) {
+    float dq[C::RT][CB][4];
+    zero<C::RT, CB>(dq);
+    rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, block_row(C::row(), a.x.L),
+                       min(C::row() + C::RT, tt.rows), 0, dq);
+    store_dq<E, C4, CB>(a, tt, b, h, dq);
   }
 }
 
-template <class T>
-static cudaError_t fwd_typed(const Launch& lc, const AttnArgs& a) {
-  dim3 grid((a.T + kWarps - 1) / kWarps, a.H, a.B);
-  launch_k(attn_fwd_simt_kernel<T>, dim3(grid), dim3(kWarps * 32), 0, lc.stream,
-
-      (const T*)a.Q, (const T*)a.K, (const T*)a.V, a.ld_qkv, (T*)a.O, a.ld_o, a.lse, a.T, a.H,
-      a.dh, a.L, 1.0f / sqrtf((float)a.dh));
-  return cudaGetLastError();
+namespace {
+template <class E>
+SimtArgs<E> simt_args(const AttnArgs& f, const AttnBwdArgs* ab) {
+  SimtArgs<E> a;
+  a.x = AttnPtrs<E>{(const E*)f.Q, (const E*)f.K, (const E*)f.V, (const E*)f.O,
+                    ab ? (const E*)ab->dO : nullptr, f.ld_qkv, f.ld_o, f.lse, f.T, f.H, f.dh, f.L,
+                    1.0f / sqrtf((float)f.dh)};
+  a.Out = (E*)f.O;
+  a.dQ = ab ? (E*)ab->dQ : nullptr;
+  a.dK = ab ? (E*)ab->dK : nullptr;
+  a.dV = ab ? (E*)ab->dV : nullptr;
+  a.ld_d = ab ? ab->ld_dqkv : 0;
+  a.lse = f.lse;
+  a.Drow = ab ? ab->Drow : nullptr;
+  a.rows = f.L <= kTile ? (kTile / f.L) * f.L : kTile;
+  a.tpb = f.L <= kTile ? 1 : (f.L + kTile - 1) / kTile;
+  // rows of q, k, v and of the gradients may have any stride; those of O and dO
+  // are D elements apart, a multiple of 64
+  a.vec = f.ld_qkv % 4 == 0 && a.ld_d % 4 == 0;
+  return a;
 }
 
-template <class T>
-static cudaError_t bwd_typed(const Launch& lc, const AttnBwdArgs& a) {
-  const AttnArgs& f = a.f;
-  dim3 grid((f.T + kWarps - 1) / kWarps, f.H, f.B);
-  const float scale = 1.0f / sqrtf((float)f.dh);
-  launch_k(attn_bwd_q_simt_kernel<T>, dim3(grid), dim3(kWarps * 32), 0, lc.stream,
-
-      (const T*)f.Q, (const T*)f.K, (const T*)f.V, f.ld_qkv, (const T*)f.O, (const T*)a.dO, f.ld_o,
-      f.lse, a.Drow, (T*)a.dQ, a.ld_dqkv, f.T, f.H, f.dh, f.L, scale);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  launch_k(attn_bwd_kv_simt_kernel<T>, dim3(grid), dim3(kWarps * 32), 0, lc.stream,
-
-      (const T*)f.Q, (const T*)f.K, (const T*)f.V, f.ld_qkv, (const T*)a.dO, f.ld_o, f.lse, a.Drow,
-      (T*)a.dK, (T*)a.dV, a.ld_dqkv, f.T, f.H, f.dh, f.L, scale);
-  return cudaGetLastError();
+// Bytes of `tiles` tiles of dh + 4 columns and `cols` columns of scores per row.
+int simt_smem(int tiles, int cols, int dh) {
+  return kTile * (tiles * (dh + 4) + cols) * (int)sizeof(float);
 }
+
+template <class K, class E, class... X>
+cudaError_t simt_launch(const Launch& lc, K kern, std::atomic<unsigned long long>* opted, int tiles,
+                        int cols, int max_cols, const AttnArgs& f, const SimtArgs<E>& a, X... x) {
+  // the limit is raised once per kernel and device, to the largest size needed
+  if (cudaError_t e = smem_opt_in(kern, simt_smem(tiles, max_cols, kMaxDh), opted);
+      e != cudaSuccess)
+    return e;
+  const int nx = f.L <= kTile ? (f.T + a.rows - 1) / a.rows : (f.T + f.L - 1) / f.L * a.tpb;
+  cudaError_t e = launch_k(kern, dim3(nx, f.H, f.B), dim3(kThreads), simt_smem(tiles, cols, f.dh),
+                           lc.stream, a, x...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// f(C4, CB) for the head width: column groups of four over 16 threads, blocks
+// of 64 columns.
+template <class F>
+cudaError_t with_cols(int dh, F&& f) {
+  using std::integral_constant;
+  if (dh <= 16) return f(integral_constant<int, 4>(), integral_constant<int, 1>());
+  if (dh <= 32) return f(integral_constant<int, 8>(), integral_constant<int, 1>());
+  if (dh <= 64) return f(integral_constant<int, 16>(), integral_constant<int, 1>());
+  return f(integral_constant<int, 16>(), integral_constant<int, 2>());
+}
+
+template <class E>
+cudaError_t fwd_typed(const Launch& lc, const AttnArgs& f) {
+  const SimtArgs<E> a = simt_args<E>(f, nullptr);
+  return with_cols(f.dh, [&](auto c4, auto cb) {
+    static std::atomic<unsigned long long> opted{0};
+    // the row's scores (four more columns of padding), and one for the sums
+    const int ldp = a.tpb <= kKeep ? a.tpb * kTile + 4 : kPld;
+    return simt_launch(lc, attn_fwd_simt_kernel<E, decltype(c4)::value, decltype(cb)::value>,
+                       &opted, 3, ldp + 1, kKeep * kTile + 5, f, a, ldp);
+  });
+}
+
+template <class E>
+cudaError_t bwd_typed(const Launch& lc, const AttnBwdArgs& ab) {
+  const SimtArgs<E> a = simt_args<E>(ab.f, &ab);
+  return with_cols(ab.f.dh, [&](auto c4, auto cb) {
+    constexpr int C4 = decltype(c4)::value, CB = decltype(cb)::value;
+    static std::atomic<unsigned long long> o1{0}, o2{0}, o3{0};
+    if (ab.f.L <= kTile)
+      return simt_launch(lc, attn_bwd_kv_simt_kernel<E, C4, CB, true>, &o1, 4, 2 * kPld, 2 * kPld, ab.f, a);
+    cudaError_t e = simt_launch(lc, attn_bwd_q_simt_kernel<E, C4, CB>, &o2, 4, kPld, kPld, ab.f, a);
+    if (e != cudaSuccess) return e;
+    return simt_launch(lc, attn_bwd_kv_simt_kernel<E, C4, CB, false>, &o3, 4, 2 * kPld, 2 * kPld, ab.f, a);
+  });
+}
+}  // namespace
 
 cudaError_t attn_fwd_simt(const Launch& lc, int dtype, const AttnArgs& a) {
   if (a.dh > kMaxDh || a.L > kMaxL) return cudaErrorInvalidValue;
