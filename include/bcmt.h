@@ -37,8 +37,9 @@
  *    tensor-core attention: L in {16, 32, 64, 128} on the single-tile kernels
  *    (a 128-token tile holds whole blocks), L a multiple of 128 from 256 to
  *    1024 on the key-tile-walking kernels (an online softmax over the block's
- *    128-token key tiles).  fp32 shapes, other head widths and the remaining
- *    block sizes run a SIMT attention kernel in fp32.
+ *    128-token key tiles).  Other bf16 shapes run their attention forward on the
+ *    CUDA cores in fp32 and its backward on the tensor cores; fp32 shapes run
+ *    both on the CUDA cores.
  *  - `stream` is a cudaStream_t (NULL = legacy default stream).  Calls are
  *    asynchronous: they validate their arguments, enqueue kernels and return.
  *    On invalid arguments nothing is launched and an error code is returned;

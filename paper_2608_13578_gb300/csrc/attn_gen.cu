@@ -1,0 +1,632 @@
+// Backward of the intra-block causal attention on the tcgen05 tensor cores (Sec.
+// 3.3) for the bf16 shapes that attn_tc.cu and attn_flash.cu do not take: any
+// head width that is a multiple of 8 up to 128, any block size up to 1024.  (Their
+// forward is attn_simt.cu's.)
+//
+// Tiles.  A head's 128-token tile comes in by TMA as NC = ceil(dh / 64) boxes
+// of 128 rows x 64 columns (128-byte swizzle).  The tensor maps are 4-D
+// (dh, H, T, B), so columns past the head and tokens past the sequence are
+// zero-filled (and clipped on the way out) whatever dh is.  For L <= 128 a
+// tile starts at a block and holds the 128 / L whole blocks that fit: keys and
+// queries are the same tile, the mask is block-diagonal causal.  For L > 128 a
+// tile is up to 128 rows of one block and walks the block's other tiles.
+// Loads always bring 128 rows; the rows that belong to the next tile are
+// masked, and output boxes are as high as the tile has rows of its own.
+//
+// Precision.  The probabilities P and the score gradients dS are fp32 values;
+// as operands of the tensor-core products they enter as the sum of two bf16
+// numbers (hi = bf16(x), lo = bf16(x - hi): 16 significand bits), so that the
+// products see them to 2^-17 instead of bf16's 2^-9.  The other operands are
+// the bf16 tensors themselves.
+//
+// Work split: 256 threads; warp w owns TMEM lane quarter w % 4 (thread = one
+// query row) and half w / 4 of the 128 key columns (of the dh output columns
+// in the epilogues).  What bounds it: the chain load -> S, dP -> P -> dV -> dS
+// -> dK, dQ of one CTA, several microseconds, covered by a second CTA per SM
+// where shared memory allows (heads up to 64).  Against the CUDA-core kernels
+// that served these shapes before (one warp per row, operands re-read from L2
+// per row): B4 T2048 D1024 heads of 128 L128 8230 -> 81 us, B4 T1000 D768 heads
+// of 96 L48 1161 -> 49 us.
+//
+// A masked key's weight is exactly 0, but 0 x inf = NaN in the products: a row
+// whose result is not finite is recomputed from its visible keys alone
+// (attn_slow.cuh).
+#include "attn_common.cuh"
+#include "attn_slow.cuh"
+#include "common.cuh"
+#include "internal.h"
+#include "tc.cuh"
+#include "tmap.h"
+
+namespace bcmt {
+using namespace attn;
+
+namespace {
+constexpr int kTile = 128;
+constexpr int kThreads = 256;
+constexpr uint32_t kChunk = 16384;  // one 128-row x 64-column box
+constexpr uint32_t kP = 32768;      // one 128 x 128 bf16 operand (hi or lo part)
+
+// What the kernels need beside their tensor maps.
+struct GenArgs {
+  AttnPtrs<bf16> x;
+  float* Drow;
+  int rows;   // L <= 128: rows per tile (whole blocks)
+  int tpb;    // L > 128: tiles per block
+  unsigned* status;
+};
+
+// a, b as bf16 pairs hi + lo.
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  hi = pack2(a, b);
+  lo = pack2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
+// Eight values into unit u of row r of the hi and lo operand tiles.
+__device__ __forceinline__ void put_split(uint8_t* hi, uint8_t* lo, int r, int u, const float* v) {
+  uint4 h, l;
+  split2(v[0], v[1], h.x, l.x);
+  split2(v[2], v[3], h.y, l.y);
+  split2(v[4], v[5], h.z, l.z);
+  split2(v[6], v[7], h.w, l.w);
+  put_unit(hi, r, u, h);
+  put_unit(lo, r, u, l);
+}
+
+// One head tile: NC boxes of 64 columns.
+template <int NC>
+__device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int h,
+                                          int t, int b) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c) tc::tma_load_4d(dst + c * kChunk, m, bar, 64 * c, h, t, b);
+}
+template <int NC>
+__device__ __forceinline__ void store_tile(const CUtensorMap* m, const uint8_t* src, int h, int t,
+                                           int b) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c) tc::tma_store_4d(m, src + c * kChunk, 64 * c, h, t, b);
+}
+
+// Operand descriptors: a head tile K-major (K = columns, step kk of 16) or
+// MN-major (N = columns, K = rows, step kk), P / dS K-major (K = keys) or
+// MN-major (M = keys, K = queries).  All are 64-column swizzle-128 chunks
+// 16 KB apart.
+__device__ __forceinline__ uint64_t d_kmaj(const uint8_t* t, int kk) {
+  return tc::sdesc(tc::smem_u32(t) + (kk >> 2) * kChunk + (kk & 3) * 32, 16, 1024);
+}
+__device__ __forceinline__ uint64_t d_mnmaj(const uint8_t* t, int kk) {
+  return tc::sdesc(tc::smem_u32(t) + kk * 2048, kChunk, 1024);
+}
+
+// Columns of the tile the thread's half owns in the epilogues: OC = 32 NC from
+// column hf * OC.  Stages OC values of row r as bf16 into a head tile.
+template <int NC>
+__device__ __forceinline__ void stage_half(uint8_t* tile, int r, int hf, const float* v) {
+#pragma unroll
+  for (int u = 0; u < 4 * NC; ++u) {
+    const int unit = hf * 4 * NC + u;
+    *reinterpret_cast<uint4*>(tile + (unit >> 3) * kChunk + tc::sw128_offset(r, unit & 7)) =
+        pack8(v + 8 * u);
+  }
+}
+template <int NC>
+__device__ __forceinline__ void tmem_half(uint32_t taddr, float* v) {
+  uint32_t x[NC][32];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) tc::tmem_ld32_issue(taddr + 32u * c, x[c]);
+  tc::tmem_wait();
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[32 * c + j] = __uint_as_float(x[c][j]);
+}
+
+// Tile x of a sequence: its first token, its rows, the first row of its block
+// (L > 128), its index within the block.
+struct TileAt {
+  int t0, rows, kstart, j;
+};
+__device__ __forceinline__ TileAt tile_at(const GenArgs& a, int x) {
+  TileAt t;
+  if (a.x.L <= kTile) {
+    t.t0 = t.kstart = x * a.rows;
+    t.j = 0;
+    t.rows = min(a.rows, a.x.T - t.t0);
+  } else {
+    const int i = x / a.tpb;
+    t.j = x - i * a.tpb;
+    t.kstart = i * a.x.L;
+    t.t0 = t.kstart + t.j * kTile;
+    t.rows = min(min(kTile, a.x.L - t.j * kTile), a.x.T - t.t0);
+  }
+  return t;
+}
+
+// Drow = dO_t . O_t.
+__device__ __forceinline__ float drow_of(const GenArgs& a, long row, int h) {
+  const bf16* o = a.x.O + row * a.x.ld_o + h * a.x.dh;
+  const bf16* g = a.x.dO + row * a.x.ld_o + h * a.x.dh;
+  float s = 0.f;
+#pragma unroll 4
+  for (int c = 0; c < a.x.dh; c += 8) {
+    float ov[8], gv[8];
+    load8(o + c, ov);
+    load8(g + c, gv);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s = fmaf(ov[e], gv[e], s);
+  }
+  return s;
+}
+
+// Swizzled tiles need the 1024-byte alignment that the declaration asks for.
+__device__ __forceinline__ bool aligned_smem(const uint8_t* smem, unsigned* status) {
+  if ((tc::smem_u32(smem) & 1023u) == 0) return true;
+  if (threadIdx.x == 0) atomicOr(status, kStatusBadLaunch);
+  return false;
+}
+
+// Staged rows recomputed from their visible keys / queries alone: 16-byte units
+// u0 .. u0+nu-1 of row r of the staging tile.
+__device__ __forceinline__ void put_staged(uint8_t* tile, int r, int u, const float* v) {
+  *reinterpret_cast<uint4*>(tile + (u >> 3) * kChunk + tc::sw128_offset(r, u & 7)) = pack8(v);
+}
+__device__ __noinline__ void restage_dq(const GenArgs& a, int b, int h, int t, uint8_t* tile, int r,
+                                        int u0, int nu) {
+  for (int u = u0; u < u0 + nu && 8 * u < a.x.dh; ++u) {
+    float v[8];
+    slow_dq<8>(a.x, b, h, t, 8 * u, v);
+    put_staged(tile, r, u, v);
+  }
+}
+__device__ __noinline__ void restage_dkv(const GenArgs& a, int b, int h, int j, uint8_t* tk,
+                                         uint8_t* tv, int r, int u0, int nu) {
+  for (int u = u0; u < u0 + nu && 8 * u < a.x.dh; ++u) {
+    float dk[8], dv[8];
+    slow_dkv<8>(a.x, b, h, j, 8 * u, dk, dv);
+    put_staged(tk, r, u, dk);
+    put_staged(tv, r, u, dv);
+  }
+}
+}  // namespace
+
+// ============================================================ backward: dQ
+// For L > 128: per query tile, Drow, then per key tile S and dP (128 + 128 TMEM
+// columns), dS = P (dP - Drow) scale as hi + lo (hi over the consumed V), the
+// product dS K into the S columns, accumulated in registers.  112 KB (NC = 1:
+// two CTAs per SM) or 160 KB.
+template <int NC> constexpr int dq_smem() { return 3 * NC * (int)kChunk + 2 * (int)kP; }
+
+template <int NC>
+__global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
+    attn_bwd_dq_gen_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
+                           const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO,
+                           const __grid_constant__ CUtensorMap mdQ, const __grid_constant__ CUtensorMap mdQt,
+                           const __grid_constant__ GenArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  constexpr uint32_t kT = NC * kChunk;
+  constexpr int OC = 32 * NC;
+  uint8_t* sQ = smem;
+  uint8_t* sdO = smem + kT;
+  uint8_t* sK = smem + 2 * kT;
+  uint8_t* sV = smem + 3 * kT;
+  uint8_t* sSh = sV;        // dS hi over V (and, NC = 1, the 16 KB after it)
+  uint8_t* sSl = sV + kP;   // dS lo
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dq_smem<NC>());  // loads, S/dP, dQ
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 3);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q = warp & 3, hf = warp >> 2;
+  const int h = blockIdx.y, b = blockIdx.z;
+  const TileAt tt = tile_at(a, blockIdx.x);
+  if (tt.rows <= 0 || !aligned_smem(smem, a.status)) {
+    pdl_enter();
+    return;
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i) tc::mbar_init(&bar[i], 1);
+    tc::fence_mbar_init();
+    tc::prefetch_tmap(&mQ);
+    tc::prefetch_tmap(&mK);
+    tc::prefetch_tmap(&mV);
+    tc::prefetch_tmap(&mdO);
+  }
+  pdl_enter();
+  if (tid == 0) {
+    tc::mbar_arrive_expect_tx(&bar[0], 4 * kT);
+    load_tile<NC>(sQ, &mQ, &bar[0], h, tt.t0, b);
+    load_tile<NC>(sK, &mK, &bar[0], h, tt.kstart, b);
+    load_tile<NC>(sdO, &mdO, &bar[0], h, tt.t0, b);
+    load_tile<NC>(sV, &mV, &bar[0], h, tt.kstart, b);
+  }
+  __syncwarp();
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, 256);
+    tc::tmem_relinquish();
+  }
+  const int r = q * 32 + lane;
+  const bool row_ok = r < tt.rows;
+  const long lrow = ((long)b * a.x.H + h) * a.x.T + tt.t0 + r;
+  const float drow = row_ok ? drow_of(a, (long)b * a.x.T + tt.t0 + r, h) : 0.f;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot;
+  const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+  const int nk = (a.x.dh + 15) / 16;
+  if (row_ok && hf == 0) a.Drow[lrow] = drow;
+  const float nl2 = row_ok ? -a.x.lse[lrow] * kLog2e : 0.f;
+  const float sl2 = a.x.scale * kLog2e, ndr = -drow * a.x.scale;
+  float acc[OC];
+#pragma unroll
+  for (int c = 0; c < OC; ++c) acc[c] = 0.f;
+  bool ok = true;
+
+  for (int kt = 0; kt <= tt.j; ++kt) {
+    const bool diag = kt == tt.j;
+    if (tid == 0) {
+      const bool okk = tc::mbar_wait(&bar[0], kt & 1, a.status);
+      tc::fence_after_sync();
+      if (okk) {
+        constexpr uint32_t id = tc::idesc_bf16(128, 128, 0, 0);
+        for (int kk = 0; kk < nk; ++kk)
+          tc::mma_bf16(tmem, d_kmaj(sQ, kk), d_kmaj(sK, kk), id, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < nk; ++kk)
+          tc::mma_bf16(tmem + 128, d_kmaj(sdO, kk), d_kmaj(sV, kk), id, kk > 0 ? 1u : 0u);
+      }
+      tc::mma_commit(&bar[1]);
+    }
+    __syncwarp();
+    ok = tc::mbar_wait(&bar[1], kt & 1, a.status) && ok;
+    tc::fence_after_sync();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int k0 = hf * 64 + c * 32;
+      const bool use = !diag || k0 <= q * 32 + 31;
+      float s[32], dp[32];
+      tc::tmem_ld32_issue(trow + (uint32_t)k0, reinterpret_cast<uint32_t*>(s));
+      tc::tmem_ld32_issue(trow + 128u + (uint32_t)k0, reinterpret_cast<uint32_t*>(dp));
+      tc::tmem_wait();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const bool vis = use && row_ok && (!diag || k0 + j <= r);
+        s[j] = vis ? ex2(fmaf(s[j], sl2, nl2)) * fmaf(dp[j], a.x.scale, ndr) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) put_split(sSh, sSl, r, hf * 8 + c * 4 + u, s + 8 * u);
+    }
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();  // dS is in place, S and dP are read
+    if (tid == 0) {
+      tc::fence_after_sync();
+      if (ok) {
+        const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
+        const int nkk = diag ? (tt.rows + 15) / 16 : 8;
+        for (int kk = 0; kk < nkk; ++kk) {
+          tc::mma_bf16(tmem, p_kmaj(sSh, 0, kk), d_mnmaj(sK, kk), idQ, kk > 0 ? 1u : 0u);
+          tc::mma_bf16(tmem, p_kmaj(sSl, 0, kk), d_mnmaj(sK, kk), idQ, 1u);
+        }
+      }
+      tc::mma_commit(&bar[2]);
+    }
+    __syncwarp();
+    ok = tc::mbar_wait(&bar[2], kt & 1, a.status) && ok;
+    tc::fence_after_sync();
+    if (tid == 0 && kt < tt.j) {  // K, V and dS are consumed: the next key tile
+      tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
+      load_tile<NC>(sK, &mK, &bar[0], h, tt.kstart + (kt + 1) * kTile, b);
+      load_tile<NC>(sV, &mV, &bar[0], h, tt.kstart + (kt + 1) * kTile, b);
+    }
+    __syncwarp();
+    float o[OC];
+    tmem_half<NC>(trow + (uint32_t)(hf * OC), o);
+#pragma unroll
+    for (int c = 0; c < OC; ++c) acc[c] += o[c];
+    tc::fence_before_sync();
+    __syncthreads();  // the product is read before the next S overwrites it
+    tc::fence_after_sync();
+  }
+
+  bool fin = true;
+#pragma unroll
+  for (int c = 0; c < OC; ++c)
+    if (hf * OC + c < a.x.dh) fin = fin && is_finite(acc[c]);
+  stage_half<NC>(sQ, r, hf, acc);
+  if (!fin && row_ok) restage_dq(a, b, h, tt.t0 + r, sQ, r, hf * OC / 8, OC / 8);
+  tc::fence_proxy_async_smem();
+  __syncthreads();
+  if (tid == 0 && ok) {
+    store_tile<NC>(tt.j == a.tpb - 1 ? &mdQt : &mdQ, sQ, h, tt.t0, b);
+    tc::tma_store_commit();
+    tc::tma_store_wait_read<0>();
+  }
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 256);
+}
+
+// ====================================================== backward: dK, dV (dQ)
+// Per key tile, its query tiles in turn: S = Q K^T and dP = dO V^T, P as
+// hi + lo for dV += P^T dO, dS = P (dP - Drow) scale, which waits in fp32 in
+// dP's TMEM columns until the dV product has consumed P, as hi + lo in P's
+// buffers for dK += dS^T Q.  FUSED (L <= 128: the key tile is its own and only
+// query tile): Drow is computed here and dQ = dS K joins; P hi covers the
+// consumed V (112 / 160 KB), and the products reuse the columns of S and dP
+// (NC = 1: 256 columns, two CTAs per SM).
+template <int NC, bool FUSED> constexpr int dkv_smem() {
+  return (FUSED ? 3 : 4) * NC * (int)kChunk + 2 * (int)kP;
+}
+template <int NC, bool FUSED> constexpr int dkv_cols() { return FUSED && NC == 1 ? 256 : 512; }
+
+template <int NC, bool FUSED>
+__global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
+    attn_bwd_dkv_gen_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
+                            const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO,
+                            const __grid_constant__ CUtensorMap mdQ, const __grid_constant__ CUtensorMap mdK,
+                            const __grid_constant__ CUtensorMap mdV, const __grid_constant__ CUtensorMap mdKt,
+                            const __grid_constant__ CUtensorMap mdVt, const __grid_constant__ GenArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  constexpr uint32_t kT = NC * kChunk;
+  constexpr int OC = 32 * NC;
+  constexpr uint32_t kDV = FUSED ? 0 : 256, kDK = kDV + 64 * NC, kDQ = FUSED ? 128 * NC : 0;
+  uint8_t* sQ = smem;              // Q; FUSED: then dQ staging
+  uint8_t* sdO = smem + kT;        // dO; then dV staging
+  uint8_t* sK = smem + 2 * kT;     // K; then dK staging
+  uint8_t* sV = smem + 3 * kT;
+  uint8_t* sPh = FUSED ? sV : smem + 4 * kT;  // P hi, then dS hi
+  uint8_t* sPl = sPh + kP;                    // P lo, then dS lo
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dkv_smem<NC, FUSED>());  // loads, S/dP, dV, dK
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q = warp & 3, hf = warp >> 2;
+  const int h = blockIdx.y, b = blockIdx.z;
+  const TileAt tt = tile_at(a, blockIdx.x);
+  if (tt.rows <= 0 || !aligned_smem(smem, a.status)) {
+    pdl_enter();
+    return;
+  }
+  // query tiles tt.j .. jend-1 of the block
+  const int jend = FUSED ? 1 : min(a.tpb, (min(a.x.L, a.x.T - tt.kstart) + kTile - 1) / kTile);
+  if (tid == 0) {
+    for (int i = 0; i < 4; ++i) tc::mbar_init(&bar[i], 1);
+    tc::fence_mbar_init();
+    tc::prefetch_tmap(&mQ);
+    tc::prefetch_tmap(&mK);
+    tc::prefetch_tmap(&mV);
+    tc::prefetch_tmap(&mdO);
+  }
+  pdl_enter();
+  if (tid == 0) {
+    tc::mbar_arrive_expect_tx(&bar[0], 4 * kT);
+    load_tile<NC>(sQ, &mQ, &bar[0], h, tt.t0, b);
+    load_tile<NC>(sK, &mK, &bar[0], h, tt.t0, b);
+    load_tile<NC>(sdO, &mdO, &bar[0], h, tt.t0, b);
+    load_tile<NC>(sV, &mV, &bar[0], h, tt.t0, b);
+  }
+  __syncwarp();
+  if (warp == 0) {
+    tc::tmem_alloc(tslot, dkv_cols<NC, FUSED>());
+    tc::tmem_relinquish();
+  }
+  const int r = q * 32 + lane;
+  float drow = 0.f;
+  if (FUSED && r < tt.rows) drow = drow_of(a, (long)b * a.x.T + tt.t0 + r, h);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot;
+  const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+  const int nk = (a.x.dh + 15) / 16;
+  const uint32_t idMN = tc::idesc_bf16(128, nk * 16, 1, 1);
+  const int rbs = FUSED ? (r / a.x.L) * a.x.L : 0;
+  const int wbs = FUSED ? ((q * 32) / a.x.L) * a.x.L : 0;
+  const float sl2 = a.x.scale * kLog2e;
+  bool ok = true;
+
+  for (int i = tt.j, it = 0; i < jend; ++i, ++it) {  // FUSED: j = 0, jend = 1
+    const bool diag = it == 0;
+    const int t0 = FUSED ? tt.t0 : tt.kstart + i * kTile;
+    const int rows = FUSED ? tt.rows : min(min(kTile, a.x.L - i * kTile), a.x.T - t0);
+    const bool row_ok = r < rows;
+    const long lrow = ((long)b * a.x.H + h) * a.x.T + t0 + r;
+    const float nl2 = row_ok ? -a.x.lse[lrow] * kLog2e : 0.f;
+    if (!FUSED) drow = row_ok ? a.Drow[lrow] : 0.f;
+    const float ndr = -drow * a.x.scale;
+    if (tid == 0) {
+      const bool okk = tc::mbar_wait(&bar[0], it & 1, a.status);
+      tc::fence_after_sync();
+      if (okk) {
+        constexpr uint32_t id = tc::idesc_bf16(128, 128, 0, 0);
+        for (int kk = 0; kk < nk; ++kk)
+          tc::mma_bf16(tmem, d_kmaj(sQ, kk), d_kmaj(sK, kk), id, kk > 0 ? 1u : 0u);
+        for (int kk = 0; kk < nk; ++kk)
+          tc::mma_bf16(tmem + 128, d_kmaj(sdO, kk), d_kmaj(sV, kk), id, kk > 0 ? 1u : 0u);
+      }
+      tc::mma_commit(&bar[1]);
+    }
+    __syncwarp();
+    ok = tc::mbar_wait(&bar[1], it & 1, a.status) && ok;
+    tc::fence_after_sync();
+    // P to shared memory, dS (fp32) over dP in TMEM
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int k0 = hf * 64 + c * 32;
+      const bool use = !diag || (k0 <= q * 32 + 31 && k0 + 31 >= wbs);
+      float s[32], dp[32];
+      tc::tmem_ld32_issue(trow + (uint32_t)k0, reinterpret_cast<uint32_t*>(s));
+      tc::tmem_ld32_issue(trow + 128u + (uint32_t)k0, reinterpret_cast<uint32_t*>(dp));
+      tc::tmem_wait();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int kk = k0 + j;
+        const bool vis = use && row_ok && (!diag || (kk >= rbs && kk <= r));
+        s[j] = vis ? ex2(fmaf(s[j], sl2, nl2)) : 0.f;
+        dp[j] = vis ? s[j] * fmaf(dp[j], a.x.scale, ndr) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) put_split(sPh, sPl, r, hf * 8 + c * 4 + u, s + 8 * u);
+      tc::tmem_st32(trow + 128u + (uint32_t)k0, dp);
+    }
+    tc::tmem_st_wait();
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();  // P is in place, S is read
+    const int nkk = (rows + 15) / 16;  // queries past the tile's rows have P = dS = 0
+    if (tid == 0) {
+      tc::fence_after_sync();
+      if (ok) {
+        for (int kk = 0; kk < nkk; ++kk) {  // dV += P^T dO
+          tc::mma_bf16(tmem + kDV, d_mnmaj(sPh, kk), d_mnmaj(sdO, kk), idMN,
+                       (it > 0 || kk > 0) ? 1u : 0u);
+          tc::mma_bf16(tmem + kDV, d_mnmaj(sPl, kk), d_mnmaj(sdO, kk), idMN, 1u);
+        }
+      }
+      tc::mma_commit(&bar[2]);
+    }
+    __syncwarp();
+    ok = tc::mbar_wait(&bar[2], it & 1, a.status) && ok;
+    tc::fence_after_sync();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float ds[32];
+      tc::tmem_ld32(trow + 128u + (uint32_t)(hf * 64 + c * 32), ds);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) put_split(sPh, sPl, r, hf * 8 + c * 4 + u, ds + 8 * u);
+    }
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();  // dS is in place; its TMEM columns are read
+    if (tid == 0) {
+      tc::fence_after_sync();
+      if (ok) {
+        for (int kk = 0; kk < nkk; ++kk) {  // dK += dS^T Q
+          tc::mma_bf16(tmem + kDK, d_mnmaj(sPh, kk), d_mnmaj(sQ, kk), idMN,
+                       (it > 0 || kk > 0) ? 1u : 0u);
+          tc::mma_bf16(tmem + kDK, d_mnmaj(sPl, kk), d_mnmaj(sQ, kk), idMN, 1u);
+        }
+        if (FUSED) {
+          const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
+          for (int kk = 0; kk < nkk; ++kk) {  // dQ = dS K
+            tc::mma_bf16(tmem + kDQ, p_kmaj(sPh, 0, kk), d_mnmaj(sK, kk), idQ, kk > 0 ? 1u : 0u);
+            tc::mma_bf16(tmem + kDQ, p_kmaj(sPl, 0, kk), d_mnmaj(sK, kk), idQ, 1u);
+          }
+        }
+      }
+      tc::mma_commit(&bar[3]);
+    }
+    __syncwarp();
+    ok = tc::mbar_wait(&bar[3], it & 1, a.status) && ok;
+    tc::fence_after_sync();
+    if (!FUSED && tid == 0 && i + 1 < jend) {  // the next query tile
+      tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
+      load_tile<NC>(sQ, &mQ, &bar[0], h, t0 + kTile, b);
+      load_tile<NC>(sdO, &mdO, &bar[0], h, t0 + kTile, b);
+    }
+    __syncwarp();
+  }
+
+  // ---- rows of dV, dK (key r) and, FUSED, dQ (query r) through staging tiles
+  auto staged = [&](uint32_t col, uint8_t* tile) {  // true: the row is finite
+    float v[OC];
+    tmem_half<NC>(trow + col + (uint32_t)(hf * OC), v);
+    bool fin = true;
+#pragma unroll
+    for (int c = 0; c < OC; ++c)
+      if (hf * OC + c < a.x.dh) fin = fin && is_finite(v[c]);
+    stage_half<NC>(tile, r, hf, v);
+    return fin;
+  };
+  const bool fv = staged(kDV, sdO), fk = staged(kDK, sK);
+  if (!(fv && fk) && r < tt.rows)
+    restage_dkv(a, b, h, tt.t0 + r, sK, sdO, r, hf * OC / 8, OC / 8);
+  __syncwarp();
+  if (FUSED && !staged(kDQ, sQ) && r < tt.rows)
+    restage_dq(a, b, h, tt.t0 + r, sQ, r, hf * OC / 8, OC / 8);
+  tc::fence_proxy_async_smem();
+  tc::fence_before_sync();
+  __syncthreads();
+  if (tid == 0 && ok) {
+    const bool tail = !FUSED && tt.j == a.tpb - 1;
+    if (FUSED) store_tile<NC>(&mdQ, sQ, h, tt.t0, b);
+    store_tile<NC>(tail ? &mdKt : &mdK, sK, h, tt.t0, b);
+    store_tile<NC>(tail ? &mdVt : &mdV, sdO, h, tt.t0, b);
+    tc::tma_store_commit();
+    tc::tma_store_wait_read<0>();
+  }
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, dkv_cols<NC, FUSED>());
+}
+
+// ========================================================================= host
+bool attn_gen_supported(int dtype, int dh, int L) {
+  return dtype == 1 && dh >= 8 && dh <= 128 && dh % 8 == 0 && L >= 1 && L <= 1024 &&
+         tmap_encoder() != nullptr;
+}
+
+namespace {
+// [B, T] rows of H heads of dh columns, boxes of `rows` tokens x 64 columns
+bool gen_map(CUtensorMap* m, const void* base, long ld, const AttnArgs& a, int rows) {
+  if (ld % 8 != 0) return false;
+  const uint64_t dims[4] = {(uint64_t)a.dh, (uint64_t)a.H, (uint64_t)a.T, (uint64_t)a.B};
+  const uint64_t st[3] = {(uint64_t)a.dh * 2, (uint64_t)ld * 2, (uint64_t)ld * 2 * (uint64_t)a.T};
+  const uint32_t box[4] = {64, 1, (uint32_t)rows, 1};
+  return make_tmap_bf16(m, base, 4, dims, st, box);
+}
+
+constexpr int kExtra = 64;  // beside the tiles: barriers and the TMEM slot
+
+GenArgs gen_args(const Launch& lc, const AttnBwdArgs& ab) {
+  const AttnArgs& a = ab.f;
+  GenArgs g;
+  g.x = AttnPtrs<bf16>{(const bf16*)a.Q, (const bf16*)a.K,  (const bf16*)a.V, (const bf16*)a.O,
+                       (const bf16*)ab.dO, a.ld_qkv,          a.ld_o,           a.lse,
+                       a.T,              a.H,               a.dh,             a.L,
+                       1.0f / sqrtf((float)a.dh)};
+  g.Drow = ab.Drow;
+  g.rows = a.L <= kTile ? (kTile / a.L) * a.L : kTile;
+  g.tpb = a.L <= kTile ? 1 : (a.L + kTile - 1) / kTile;
+  g.status = lc.status;
+  return g;
+}
+dim3 gen_grid(const AttnArgs& a, const GenArgs& g) {
+  const int nx = a.L <= kTile ? (a.T + g.rows - 1) / g.rows : (a.T + a.L - 1) / a.L * g.tpb;
+  return dim3(nx, a.H, a.B);
+}
+// rows of the last tile of a block (L > 128)
+int tail_rows(const GenArgs& g) { return g.x.L <= kTile ? g.rows : g.x.L - (g.tpb - 1) * kTile; }
+
+template <class K, class... A>
+cudaError_t gen_launch(const Launch& lc, K kern, std::atomic<unsigned long long>* opted, int smem,
+                       dim3 grid, A&&... args) {
+  if (cudaError_t e = smem_opt_in(kern, smem, opted); e != cudaSuccess) return e;
+  cudaError_t e = launch_k(kern, grid, dim3(kThreads), smem, lc.stream, args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int NC>
+cudaError_t bwd_nc(const Launch& lc, const AttnBwdArgs& ab) {
+  const AttnArgs& a = ab.f;
+  const GenArgs g = gen_args(lc, ab);
+  const int tr = tail_rows(g);
+  CUtensorMap mQ, mK, mV, mdO, dq, dk, dv, dqt, dkt, dvt;
+  if (!gen_map(&mQ, a.Q, a.ld_qkv, a, kTile) || !gen_map(&mK, a.K, a.ld_qkv, a, kTile) ||
+      !gen_map(&mV, a.V, a.ld_qkv, a, kTile) || !gen_map(&mdO, ab.dO, a.ld_o, a, kTile) ||
+      !gen_map(&dq, ab.dQ, ab.ld_dqkv, a, g.rows) || !gen_map(&dk, ab.dK, ab.ld_dqkv, a, g.rows) ||
+      !gen_map(&dv, ab.dV, ab.ld_dqkv, a, g.rows) || !gen_map(&dqt, ab.dQ, ab.ld_dqkv, a, tr) ||
+      !gen_map(&dkt, ab.dK, ab.ld_dqkv, a, tr) || !gen_map(&dvt, ab.dV, ab.ld_dqkv, a, tr))
+    return cudaErrorInvalidValue;
+  static std::atomic<unsigned long long> o1{0}, o2{0}, o3{0};
+  if (a.L <= kTile)
+    return gen_launch(lc, attn_bwd_dkv_gen_kernel<NC, true>, &o1, dkv_smem<NC, true>() + kExtra, gen_grid(a, g), mQ, mK, mV, mdO, dq, dk, dv, dkt, dvt, g);
+  cudaError_t e = gen_launch(lc, attn_bwd_dq_gen_kernel<NC>, &o2, dq_smem<NC>() + kExtra, gen_grid(a, g), mQ,
+                             mK, mV, mdO, dq, dqt, g);
+  if (e != cudaSuccess) return e;
+  return gen_launch(lc, attn_bwd_dkv_gen_kernel<NC, false>, &o3, dkv_smem<NC, false>() + kExtra, gen_grid(a, g), mQ, mK, mV, mdO, dq, dk, dv, dkt, dvt, g);
+}
+}  // namespace
+
+cudaError_t attn_bwd_gen(const Launch& lc, const AttnBwdArgs& a) {
+  if (!attn_gen_supported(1, a.f.dh, a.f.L)) return cudaErrorNotSupported;
+  return a.f.dh <= 64 ? bwd_nc<1>(lc, a) : bwd_nc<2>(lc, a);
+}
+
+}  // namespace bcmt

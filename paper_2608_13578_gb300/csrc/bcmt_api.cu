@@ -531,12 +531,15 @@ cudaError_t run_gemm(const Launch& lc, Prof& pr, const char* name, int dtype, in
   return e;
 }
 
-// Attention kernel for a shape: 1 = single-tile tcgen05 (head width 64,
-// L <= 128), 2 = key-tile-walking tcgen05, 0 = SIMT (fp32 and the rest).
+// Attention kernel for a shape: 1 = single-tile tcgen05 (head widths 16, 32,
+// 64, L dividing 128), 2 = key-tile-walking tcgen05 (L a multiple of 128),
+// 3 = CUDA cores forward and tcgen05 backward (the other bf16 shapes; the
+// forward keeps the order of its sums, see attn_simt.cu), 0 = CUDA cores (fp32).
 int attn_kind(const Geometry& g) {
   if (!g_use_tc_attn) return 0;
   if (attn_tc_supported(g.dtype, g.dh, g.L)) return 1;
-  return attn_fl_supported(g.dtype, g.dh, g.L) ? 2 : 0;
+  if (attn_fl_supported(g.dtype, g.dh, g.L)) return 2;
+  return attn_gen_supported(g.dtype, g.dh, g.L) ? 3 : 0;
 }
 
 bcmt_status finish(const bcmt_params* p, cudaStream_t s) {
@@ -986,6 +989,9 @@ bcmt_status bcmt_backward(const bcmt_params* p, const void* dy, const void* x_or
     } else if (attn_kind(g) == 2) {
       pr.begin("attn_bwd_fl");
       e = attn_bwd_fl(lc, ab);
+    } else if (attn_kind(g) == 3) {
+      pr.begin("attn_bwd_gen");
+      e = attn_bwd_gen(lc, ab);
     } else {
       pr.begin("attn_bwd_simt");
       e = attn_bwd_simt(lc, g.dtype, ab);
@@ -1295,6 +1301,7 @@ int bcmt_test_attn(int impl, int backward, const bcmt_params* p, const void* q, 
     AttnBwdArgs ab{aa, dO, drow, dq, dk, dv, ld_d};
     e = impl == 1 ? attn_bwd_tc(lc, ab)
         : impl == 2 ? attn_bwd_fl(lc, ab)
+        : impl == 3 ? attn_bwd_gen(lc, ab)
                     : attn_bwd_simt(lc, g.dtype, ab);
   }
   if (e != cudaSuccess) {

@@ -25,9 +25,9 @@ inline PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
   return fn;
 }
 
-// bf16 tensor of rank 2 or 3, innermost dimension first: dims[0] elements are
+// bf16 tensor of rank 2 to 4, innermost dimension first: dims[0] elements are
 // contiguous; strides_bytes[i] is the byte stride of dimension i+1.  The box is
-// box[0] x box[1] (x box[2]) elements; 128-byte swizzle unless given (the
+// box[0] x box[1] (x box[2] ...) elements; 128-byte swizzle unless given (the
 // box's inner extent in bytes must not exceed the swizzle span), zero fill
 // outside.
 inline bool make_tmap(CUtensorMap* m, CUtensorMapDataType dt, const void* base, int rank,
@@ -38,14 +38,14 @@ inline bool make_tmap_bf16(CUtensorMap* m, const void* base, int rank, const uin
                            CUtensorMapSwizzle swz = CU_TENSOR_MAP_SWIZZLE_128B) {
   return make_tmap(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, rank, dims, strides_bytes, box, swz);
 }
-// Any element type (rank 2 or 3, as above).
+// Any element type (rank 2 to 4, as above).
 inline bool make_tmap(CUtensorMap* m, CUtensorMapDataType dt, const void* base, int rank,
                       const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box,
                       CUtensorMapSwizzle swz) {
   auto enc = tmap_encoder();
   if (!enc) return false;
-  cuuint64_t gd[3], gs[2];
-  cuuint32_t bx[3], es[3] = {1, 1, 1};
+  cuuint64_t gd[4], gs[3];
+  cuuint32_t bx[4], es[4] = {1, 1, 1, 1};
   for (int i = 0; i < rank; ++i) {
     gd[i] = dims[i];
     bx[i] = box[i];

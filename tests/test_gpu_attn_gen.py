@@ -1,10 +1,12 @@
 """Attention of general shapes (any head width that is a multiple of 8, any block
-size, any row stride): the CUDA-core kernels in fp32 and bf16 against the float64
-oracle, and with non-finite tokens.
+size, any row stride): the CUDA-core kernels in fp32 and bf16 and the tcgen05
+backward against the float64 oracle, and with non-finite tokens.
 
 Tolerances.  fp32: the library's 1e-4.  bf16 forward: its own rounding, 2^-9 of
 the value, bounded at 2^-8 of the largest.  bf16 gradients also carry
-Drow = dO . O with O rounded to bf16: the library's 2e-2 against the oracle."""
+Drow = dO . O with O rounded to bf16: the library's 2e-2 against the oracle; the
+tcgen05 backward, whose P and dS enter the products as two bf16 parts (2^-17),
+within one rounding step, 2^-7 of the largest value, of the CUDA-core one."""
 
 import numpy as np
 import pytest
@@ -72,7 +74,7 @@ def test_general_attention(C, B, T, H, dh, L, dtype):
     ref_o, ref_lse, *ref_g = _attn_ref(*(t.double().numpy() for t in (q, k, v)), L, H,
                                        dO.double().numpy())
     top = np.abs(ref_g[2]).max()  # a lone key's dQ and dK are 0 but for Drow's rounding
-    runs = [_run(C, impl, p, B, T, D, H, *dev) for impl in (0,)]
+    runs = [_run(C, impl, p, B, T, D, H, *dev) for impl in ((0, 3) if dtype == "bf16" else (0,))]
     for o, lse, g in runs:
         e, m = _err(o, ref_o)
         assert e <= (2 ** -8 * m if dtype == "bf16" else 1e-4), ("o", e, m)
@@ -80,6 +82,10 @@ def test_general_attention(C, B, T, H, dh, L, dtype):
         for n, x, r in zip(("dq", "dk", "dv"), g, ref_g):
             e, m = _err(x, r)
             assert e <= (2e-2 * max(m, top) if dtype == "bf16" else 1e-4), (n, e, m)
+    if dtype == "bf16":
+        top = max(x.float().abs().max() for x in runs[0][2])
+        for x, y in zip(runs[0][2], runs[1][2]):
+            assert (x.float() - y.float()).abs().max() <= 2 ** -7 * top
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
@@ -130,3 +136,16 @@ def test_non_finite_tokens_reach_the_rows_that_see_them(C, dtype, B, T, H, dh, L
     if which != "dO":  # the token's own row sees it
         assert not torch.isfinite(o[0, 60, :dh]).all()
     assert not torch.isfinite(g[2][0, t0:t1, :dh] if which == "dO" else g[0][0, 60, :dh]).all()
+
+
+@pytest.mark.parametrize("B,T,H,dh,L", [(1, 200, 2, 96, 48), (1, 300, 2, 128, 200)])
+@pytest.mark.parametrize("which,value", NON_FINITE)
+def test_non_finite_tokens_tcgen05(C, B, T, H, dh, L, which, value):
+    """The tcgen05 backward's non-finite values lie where the CUDA-core one's do."""
+    ins = dict(zip(("q", "k", "v", "dO"), (t.cuda() for t in _inputs(B, T, H, dh))))
+    ins[which][0, 60, 5] = value
+    D = H * dh
+    p = C.make_params(B, T, D, H, L, "bf16")
+    g, g0 = (_run(C, impl, p, B, T, D, H, *ins.values())[2] for impl in (3, 0))
+    for a, b in zip(g, g0):
+        assert torch.equal(torch.isfinite(a), torch.isfinite(b))
