@@ -278,9 +278,30 @@ int device_sms() {
 bool dw_pair(int dtype, int M, int N) {
   return dtype == BCMT_BF16 && g_use_tc_gemm && M % 256 == 0 && N % 256 == 0;
 }
+// fp32 tensors on the split-bf16 tensor-core product (gemm_f32).
+bool tc_f32(int dtype) { return dtype == BCMT_F32 && g_use_tc_gemm && gemm_tc_available(); }
+
 int dw_splits(int dtype, int M, int N, long K, int max_pairs = 0) {
   const int nkb = (int)((K + 63) / 64);
   int target, tiles;
+  if (tc_f32(dtype)) {
+    // 128 x 128 tiles, one CTA per SM: the count whose waves of slices (about
+    // 1.1 us each, two more per tile to fill and store) and partials (written
+    // and read once, 5 MB per us) take the least time
+    const long t = (long)((M + 127) / 128) * ((N + 127) / 128);
+    const int sms = device_sms(), smax = std::max(1, std::min(16, nkb / 8));
+    int best = 1;
+    double best_t = -1.0;
+    for (int s = 1; s <= smax; ++s) {
+      const long waves = (t * s + sms - 1) / sms;
+      const double us = waves * ((nkb + s - 1) / s + 2) * 1.1 + s * (double)M * N * 8.0 / 5e6;
+      if (best_t < 0 || us < best_t) {
+        best_t = us;
+        best = s;
+      }
+    }
+    return best;
+  }
   if (dw_pair(dtype, M, N)) {
     tiles = (M / 256) * (N / 256);
     target = tiles >= 8 ? device_sms() / 2 : std::min(50, 12 * tiles);
@@ -506,6 +527,8 @@ cudaError_t weight_grad(const Launch& lc, Prof& pr, const char* name, int dtype,
           ? gemm_tc_pair(lc, 0, M, N, (int)K, A, 1, lda, B, ldb, 1, EPI_PARTIAL, ea, splits)
       : (dtype == 1 && g_use_tc_gemm)
           ? gemm_tc(lc, 0, M, N, (int)K, A, 1, lda, B, ldb, 1, EPI_PARTIAL, ea, splits)
+      : tc_f32(dtype)
+          ? gemm_f32(lc, M, N, (int)K, A, 1, lda, B, ldb, 1, EPI_PARTIAL, ea, splits)
           : gemm_simt(lc, dtype, 0, M, N, (int)K, A, 1, lda, B, ldb, 1, EPI_PARTIAL, ea, splits);
   pr.end(nullptr);
   if (e != cudaSuccess) return e;
@@ -526,6 +549,8 @@ cudaError_t run_gemm(const Launch& lc, Prof& pr, const char* name, int dtype, in
   cudaError_t e =
       (dtype == 1 && g_use_tc_gemm)
           ? gemm_tc(lc, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, epi, ea, splits)
+      : tc_f32(dtype)
+          ? gemm_f32(lc, M, N, K, A, sam, sak, B, sbk, sbn, epi, ea, splits)
           : gemm_simt(lc, dtype, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, epi, ea, splits);
   pr.end(nullptr);
   return e;
@@ -694,7 +719,7 @@ bcmt_status bcmt_forward(const bcmt_params* p, const void* x, const void* q, con
   // Sec. 3.3: H = Concat(heads) W_O (HOnly: this is the output, Sec. 4.5).  The
   // epilogue also forms partial pooling scores H w_p over each run of columns
   // it stores (32 columns per tcgen05 TMEM load, 4 per SIMT thread).
-  const int npart = D / ((g.dtype == BCMT_BF16 && g_use_tc_gemm) ? 32 : 4);
+  const int npart = D / ((g.dtype == BCMT_BF16 ? g_use_tc_gemm : tc_f32(g.dtype)) ? 32 : 4);
   if (fuse) {
     // H and the gate G = sigmoid(H W_g) (Sec. 3.8) in one product over all
     // SMs, [H | U] = Concat [W_O | W_O W_g]
@@ -1243,12 +1268,17 @@ int bcmt_test_gemm(int impl, int dtype, int dtype_out, int M, int N, int K, cons
   ea.ldo = ldc;
   ea.split_stride = (long)M * ldc;
   const EpiKind ek = splits > 1 ? EPI_PARTIAL : EPI_STORE;
+  if (impl == 6 && (dtype != BCMT_F32 || dtype_out != BCMT_F32)) {
+    fail(BCMT_ERR_ARG, "test gemm: impl 6 takes and gives fp32");
+    return -1;
+  }
   // impl 3, 4, 5: the single-CTA kernel with 128-, 256- or 64-wide tiles
   g_force_bn = impl == 3 ? 128 : impl == 4 ? 256 : impl == 5 ? 64 : 0;
   cudaError_t e =
-      (impl == 1 || impl >= 3)
+      (impl == 1 || (impl >= 3 && impl <= 5))
           ? gemm_tc(lc, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, ek, ea, splits)
       : impl == 2 ? gemm_tc_pair(lc, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, ek, ea, splits)
+      : impl == 6 ? gemm_f32(lc, M, N, K, A, sam, sak, B, sbk, sbn, ek, ea, splits)
                   : gemm_simt(lc, dtype, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, ek, ea,
                               splits);
   g_force_bn = 0;

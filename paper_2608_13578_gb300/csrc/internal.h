@@ -81,6 +81,14 @@ cudaError_t gemm_simt(const Launch& lc, int dtype, int dtype_out, int M, int N, 
                       const void* A, long sam, long sak, const void* B, long sbk, long sbn,
                       EpiKind epi, const EpiArgs& ea, int splits);
 
+// The same product of fp32 tensors on the tensor cores, to fp32 accuracy (each
+// operand as three bf16 parts).  EPI_STORE, EPI_PARTIAL, and for K-major A and
+// N-major B EPI_GATE and EPI_STORE_SCORE (n = 32 columns); cudaErrorNotSupported
+// for operands that cannot be read in 16-byte pieces.
+cudaError_t gemm_f32(const Launch& lc, int M, int N, int K, const void* A, long sam, long sak,
+                     const void* B, long sbk, long sbn, EpiKind epi, const EpiArgs& ea,
+                     int splits);
+
 // tcgen05 GEMM (bf16 inputs, fp32 TMEM accumulation).  A must be either
 // K-major (sak == 1) or M-major (sam == 1), B either K-major (sbk == 1) or
 // N-major (sbn == 1).  Returns cudaErrorNotSupported for other layouts.
