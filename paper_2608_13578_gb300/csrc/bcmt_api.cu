@@ -1086,8 +1086,8 @@ DecodeState decode_layout(const Geometry& g, void* base, size_t* bytes) {
   st.hhat = f32(bd);
   st.H = f32(bd);
   st.U = f32(bd);
-  st.pm = f32(g.B);
-  st.pden = f32(g.B);
+  st.pm = f32(2 * (size_t)g.B);
+  st.pden = f32(2 * (size_t)g.B);
   st.pnum = f32(bd);
   st.N = f32(bd);
   st.Z = f32(bd);
@@ -1148,7 +1148,7 @@ bcmt_status bcmt_decode_step(const bcmt_params* p, void* state, long pos, const 
   a.L = g.L;
   a.j = (int)(pos % g.L);
   a.honly = g.honly;
-  a.x = a.s.xf;
+  a.x_t = x_t;
   a.w_qkv = w_qkv;
   a.w_o = w_o;
   a.w_p = w_p;
@@ -1156,8 +1156,7 @@ bcmt_status bcmt_decode_step(const bcmt_params* p, void* state, long pos, const 
   a.w_g = w_g;
   a.decay = decay;
   a.y = y_t;
-  cudaError_t e = decode_widen(lc, g.dtype, x_t, a.s.xf, (long)g.B * g.D);
-  if (e == cudaSuccess) e = decode_step(lc, g.dtype, a);
+  cudaError_t e = decode_step(lc, g.dtype, a);
   if (e != cudaSuccess) return cuda_fail(e, "decode step");
   return finish(p, lc.stream);
 }

@@ -260,7 +260,8 @@ cudaError_t fill_zero(const Launch& lc, void* p, size_t bytes);
 struct DecodeState {
   void *Kc, *Vc;                    // [B, L, D] storage dtype
   float *xf, *qkv, *hhat, *H, *U;   // step temporaries: [B, D], [B, 3D], [B, D] x3
-  float *pm, *pden;                 // [B]: running max and denominator of the block's scores
+  float *pm, *pden;                 // [2][B]: running max and denominator of the block's scores
+                                    // (the one-launch step alternates between the two)
   float *pnum;                      // [B, D]: running numerator sum exp(s - m) H
   float *N, *Z;                     // [B, D]: N_i, Z_i of the last completed block
   float *C;                         // [B, D]: memory row of the current block
@@ -269,13 +270,12 @@ struct DecodeState {
 struct DecodeArgs {
   int B, D, H, dh, L, j;  // j = slot of the token in its block
   bool honly;
-  const float* x;         // the token's input rows, fp32 [B, D]
+  const void* x_t;        // the token's input rows [B, D], storage dtype
   const void *w_qkv, *w_o, *w_p, *w_m, *w_g;
   const float* decay;
   void* y;                // [B, D] storage dtype
   DecodeState s;
 };
-cudaError_t decode_widen(const Launch& lc, int dtype, const void* x, float* out, long n);
 cudaError_t decode_step(const Launch& lc, int dtype, const DecodeArgs& a);
 
 }  // namespace bcmt
