@@ -15,6 +15,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -1042,6 +1044,59 @@ cudaError_t gemm_tc_pair(const Launch& lc, int dtype_out, int M, int N, int K, c
 bool tc2_group_schedule(const Tc2Shape* shape, int count, int max_pairs,
                         std::vector<std::vector<int>>* lists, long* makespan);
 
+// The schedule of a group as the kernel takes it.  It depends on the products'
+// tile counts alone and takes about 15 us to work out (some 200 items onto 76
+// pairs), so the last kSchedKept shapes' schedules are kept.
+struct Tc2Schedule {
+  int npairs = 0;  // 0: round-robin
+  uint16_t start[kTc2SchedPairs + 1];
+  uint16_t list[kTc2SchedItems];
+};
+constexpr size_t kSchedKept = 32;
+template <class Op0, class Op1>
+static void tc2_schedule(Tc2Params<Op0, Op1>* P) {
+  std::array<int, 1 + 5 * kTc2Max> key{};
+  key[0] = sm_count() / 2;
+  for (int q = 0; q < P->count; ++q) {
+    const Tc2Shape& s = P->shape[q];
+    const int v[5] = {s.kps, s.nkb, s.tiles_m, s.tiles_n, s.n_tiles};
+    std::copy(v, v + 5, key.begin() + 1 + 5 * q);
+  }
+  static std::mutex mu;
+  static std::vector<std::pair<std::array<int, 1 + 5 * kTc2Max>, Tc2Schedule>> kept;
+  static size_t next = 0;  // the entry to replace when all are taken
+  std::lock_guard<std::mutex> lock(mu);
+  const Tc2Schedule* found = nullptr;
+  for (const auto& e : kept)
+    if (e.first == key) found = &e.second;
+  if (!found) {
+    Tc2Schedule s;
+    std::vector<std::vector<int>> lists;
+    if (tc2_group_schedule(P->shape, P->count, key[0], &lists, nullptr)) {
+      s.npairs = (int)lists.size();
+      int k = 0;
+      for (int p = 0; p < s.npairs; ++p) {
+        s.start[p] = (uint16_t)k;
+        for (int item : lists[p]) s.list[k++] = (uint16_t)item;
+      }
+      s.start[s.npairs] = (uint16_t)k;
+    }
+    if (kept.size() < kSchedKept) {
+      kept.emplace_back(key, s);
+      found = &kept.back().second;
+    } else {
+      kept[next] = {key, s};
+      found = &kept[next].second;
+      next = (next + 1) % kSchedKept;
+    }
+  }
+  P->npairs_sched = found->npairs;
+  if (found->npairs) {
+    memcpy(P->start, found->start, sizeof(P->start));
+    memcpy(P->list, found->list, sizeof(P->list));
+  }
+}
+
 cudaError_t gemm_tc_pair_group(const Launch& lc, const PairProduct& p0, const PairProduct* w,
                                int nw) {
   if (nw < 1 || nw > kTc2Max - 1) return cudaErrorInvalidValue;
@@ -1076,16 +1131,7 @@ cudaError_t gemm_tc_pair_group(const Launch& lc, const PairProduct& p0, const Pa
   }
   P.count = 1 + nw;
   // the pairs' item lists, longest first onto the least loaded pair
-  std::vector<std::vector<int>> lists;
-  if (tc2_group_schedule(P.shape, P.count, sm_count() / 2, &lists, nullptr)) {
-    P.npairs_sched = (int)lists.size();
-    int k = 0;
-    for (int p = 0; p < P.npairs_sched; ++p) {
-      P.start[p] = (uint16_t)k;
-      for (int item : lists[p]) P.list[k++] = (uint16_t)item;
-    }
-    P.start[P.npairs_sched] = (uint16_t)k;
-  }
+  tc2_schedule(&P);
   return tc2_run<256, ST, ACC, Op0, Op1>(lc, P);
 }
 
@@ -1116,16 +1162,7 @@ cudaError_t gemm_tc_pair_two(const Launch& lc, int M, int N, int K, const void* 
   P.shape[0] = tc2_shape<256>(M, N, K, 1);
   P.shape[1] = tc2_shape<256>(p1.M, p1.N, p1.K, 1);
   P.count = 2;
-  std::vector<std::vector<int>> lists;
-  if (tc2_group_schedule(P.shape, P.count, sm_count() / 2, &lists, nullptr)) {
-    P.npairs_sched = (int)lists.size();
-    int k = 0;
-    for (int q = 0; q < P.npairs_sched; ++q) {
-      P.start[q] = (uint16_t)k;
-      for (int item : lists[q]) P.list[k++] = (uint16_t)item;
-    }
-    P.start[P.npairs_sched] = (uint16_t)k;
-  }
+  tc2_schedule(&P);
   return tc2_run<256, ST, ACC, Op, Op>(lc, P);
 }
 

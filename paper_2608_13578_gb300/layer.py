@@ -30,14 +30,15 @@ def forward(p, t: Dict[str, torch.Tensor], stream=None, workspace: Optional[torc
     """Runs bcmt_forward on the tensors in ``t`` (keys as in ``inputs.make_inputs``).
 
     Returns (y, workspace)."""
-    ref = t["x"] if p.input_is_x else t["q"]
+    from_x = p.input_is_x
+    x = t["x"] if from_x else None
+    q, k, v = (None, None, None) if from_x else (t["q"], t["k"], t["v"])
+    ref = x if from_x else q
     y = torch.empty_like(ref)
     if workspace is None:
         workspace = _buffer(C.bcmt_workspace_size(p), ref.device)
-    C.bcmt_forward(p, t.get("x") if p.input_is_x else None,
-                   None if p.input_is_x else t["q"], None if p.input_is_x else t["k"],
-                   None if p.input_is_x else t["v"], t.get("w_qkv") if p.input_is_x else None,
-                   t["w_o"], t["w_p"], t["w_m"], t["w_g"], t["decay"], y, workspace, stream)
+    C.bcmt_forward(p, x, q, k, v, t.get("w_qkv") if from_x else None, t["w_o"], t["w_p"],
+                   t["w_m"], t["w_g"], t["decay"], y, workspace, stream)
     return y, workspace
 
 
@@ -46,26 +47,21 @@ def backward(p, t: Dict[str, torch.Tensor], workspace: torch.Tensor, dy: torch.T
              decay_grad: bool = False):
     """Runs bcmt_backward; returns a dict of gradients (dx or dq/dk/dv, dw_*, and
     d_decay when ``decay_grad``)."""
-    dev = dy.device
     if scratch is None:
-        scratch = _buffer(C.bcmt_scratch_size(p), dev)
-    g = out if out is not None else {}
-    if p.input_is_x:
-        g.setdefault("dx", torch.empty_like(t["x"]))
-        g.setdefault("dw_qkv", torch.empty_like(t["w_qkv"]))
-    else:
-        for n in ("dq", "dk", "dv"):
-            g.setdefault(n, torch.empty_like(t[n[1]]))
-    for n in ("w_o", "w_p", "w_m", "w_g"):
-        g.setdefault("d" + n, torch.empty_like(t[n]))
+        scratch = _buffer(C.bcmt_scratch_size(p), dy.device)
+    from_x = p.input_is_x
+    like = {"dx": "x", "dw_qkv": "w_qkv"} if from_x else {"dq": "q", "dk": "k", "dv": "v"}
+    like.update(dw_o="w_o", dw_p="w_p", dw_m="w_m", dw_g="w_g")
     if decay_grad:
-        g.setdefault("d_decay", torch.empty_like(t["decay"]))
-    C.bcmt_backward(p, dy, t["x"] if p.input_is_x else t["q"],
-                    None if p.input_is_x else t["k"], None if p.input_is_x else t["v"],
-                    t.get("w_qkv") if p.input_is_x else None, t["w_o"], t["w_p"], t["w_m"],
-                    t["w_g"], t["decay"], workspace, scratch,
-                    g["dx"] if p.input_is_x else g["dq"], None if p.input_is_x else g["dk"],
-                    None if p.input_is_x else g["dv"], g.get("dw_qkv"), g["dw_o"], g["dw_p"],
+        like["d_decay"] = "decay"
+    g = out if out is not None else {}
+    for n, src in like.items():
+        if n not in g:
+            g[n] = torch.empty_like(t[src])
+    x, k, v, w_qkv = (t["x"], None, None, t["w_qkv"]) if from_x else (t["q"], t["k"], t["v"], None)
+    dx, dk, dv = (g["dx"], None, None) if from_x else (g["dq"], g["dk"], g["dv"])
+    C.bcmt_backward(p, dy, x, k, v, w_qkv, t["w_o"], t["w_p"], t["w_m"], t["w_g"], t["decay"],
+                    workspace, scratch, dx, dk, dv, g.get("dw_qkv"), g["dw_o"], g["dw_p"],
                     g["dw_m"], g["dw_g"], stream, g.get("d_decay"))
     return g
 
@@ -118,7 +114,7 @@ class Decoder:
     def step(self, x_t: torch.Tensor, stream=None) -> torch.Tensor:
         w = self.w
         x_t = x_t.contiguous()
-        y = torch.empty(x_t.shape, dtype=x_t.dtype, device=x_t.device)
+        y = torch.empty_like(x_t)
         C.bcmt_decode_step(self.p, self.state, self.pos, x_t, w["w_qkv"], w["w_o"],
                            w.get("w_p"), w.get("w_m"), w.get("w_g"), w.get("decay"), y, stream)
         self.pos += 1
