@@ -15,16 +15,17 @@
 // One CTA per SM walks 128 x BN output tiles.  Warps 0-7 bring fp32 operands
 // from global memory into registers a slice ahead, split them and write the
 // three bf16 parts to a two-stage shared ring in the 128-byte-swizzled operand
-// layout (K-major or MN-major, whichever way the operand lies in memory); warp
-// 0 issues each slice's MMAs once all eight have written it (a warp of its own
-// for that would cost every thread a quarter of its registers); warps 8-15
-// drain the accumulators (two, alternating) and store finished tiles through
-// shared memory with TMA.  8192 x 1536 x 512 takes 122 us (106 TFLOP/s of fp32
-// products), 512 x 1536 x 8192 in 3 splits 112 us; the CUDA-core kernel took 497
-// and 749 us.  A 64-deep slice of a 128 x 128 tile is 1536 cycles of tensor work
-// and 2300 of shared-memory traffic (96 KB of parts written, 192 KB read by the
-// 24 MMAs); it takes about 5500, the loaders' splitting and the hand-over
-// between the two stages.
+// layout (K-major or MN-major, whichever way the operand lies in memory); warps
+// 8-15 drain the accumulators (two, alternating) and store finished tiles through
+// shared memory with TMA; warp 8 also issues the MMAs, one slice ahead of its
+// draining (a warp of its own for that would cost every thread a quarter of its
+// registers, and a loader that issues them holds up all the splitting).8192 x 1536 x 512 takes 96 us
+// (134 TFLOP/s of fp32 products; 122 us with a loader warp issuing the MMAs),
+// 512 x 1536 x 8192 in 3 splits 80 us (112); the CUDA-core kernel took 497 and
+// 749 us.  A 64-deep slice of a 128 x 128 tile is 1536 cycles of tensor work and
+// 2300 of shared-memory traffic (96 KB of parts written, 192 KB read by the 24
+// MMAs); it takes about 4000, the splitting and the hand-over between the two
+// stages.
 //
 // A row or column holding an infinity (or a value above bf16's range) makes
 // partial products like inf x 0: outputs that come out non-finite are
@@ -299,10 +300,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&full[s]);
-        if (warp == 0) {
-          if (lane == 0) ok = issue(it);
-          ok = __shfl_sync(0xffffffffu, ok, 0);
-        }
       }
       tile += gridDim.x;
       if (tile < n_tiles) tile_at(tile, m0, n0, z, kb, ke);
@@ -313,7 +310,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3, c_beg = ((warp - 8) >> 2) * NC;
     uint8_t* sbuf = smem + C::OUT_OFF + (warp - 8) * 4096;
     const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c_beg;
-    int it = 0;
+    int it = 0, slices = 0;  // warp 8 also issues the MMAs, a slice ahead of its draining
+    if (warp == 8)
+      for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        int m0, n0, z, kb, ke;
+        tile_at(tile, m0, n0, z, kb, ke);
+        slices += (ke - kb + kBK - 1) / kBK;
+      }
+    if (slices > 0 && lane == 0) issue(0);
+    __syncwarp();
     bool ok = true;
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       int m0, n0, z, kb, ke;
@@ -323,6 +328,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < NC; ++c) acc[c] = 0.f;
       for (int k = kb; k < ke; k += kBK, ++it) {
         const int ab = it & 1, use = it >> 1;
+        if (it + 1 < slices && lane == 0) issue(it + 1);
+        __syncwarp();
         ok = tc::mbar_wait(&tfull[ab], use & 1, status) && ok;
         tc::fence_after_sync();
 #pragma unroll
