@@ -15,9 +15,10 @@
 // have outputs at every head width, and skips what the causal mask hides from
 // its rows.  Bound: fp32 issue, shared-memory bandwidth close behind.  Before,
 // one warp per query row read every key row from L2; times before and now:
-// B8 T1024 D512 h8 L64 fp32 forward 516 and 59 us, backward 2002 and 120 us;
-// B4 T2048 D1024 h8 L128 bf16 forward 1997 and 172 us; B4 T1000 D768 h8 L48 bf16
-// forward 306 and 61 us.  Deterministic: every sum runs in a fixed order.
+// B8 T1024 D512 h8 L64 fp32 forward 516 and 59 us, backward 2002 and 93 us;
+// B4 T2048 D1024 h8 L128 bf16 forward 1997 and 131 us; B4 T1000 D768 h8 L48 bf16
+// forward 306 and 63 us.  Deterministic: every sum runs in a fixed order.
+#include <algorithm>
 #include <mutex>
 
 #include "attn_slow.cuh"
@@ -173,7 +174,9 @@ struct Cols {
   __device__ __forceinline__ static int row() { return (threadIdx.x / C4) * RT; }
 };
 
-// acc[i] += sum over keys j in [lo, hi), in order, of P[row + i][j] B[j - b0].
+// acc[i] += sum over keys j in [lo, hi), in order, of P[row + i][j] B[j - b0], four
+// keys at a time: the range is widened to multiples of four, where P is 0 (hidden
+// keys) and B has its zero rows.
 template <int C4, int CB>
 __device__ __forceinline__ void rows_times(const float* P, int ldp, const float* B, int ldh, int dh,
                                            int lo, int hi, int b0, float (*acc)[CB][4]) {
@@ -181,23 +184,28 @@ __device__ __forceinline__ void rows_times(const float* P, int ldp, const float*
   const float* p = P + C::row() * ldp;
   const int c = C::col();
   if (c >= dh) return;
-#pragma unroll 4
-  for (int j = lo; j < hi; ++j) {
-    float w[C::RT];
+#pragma unroll 2
+  for (int j = lo & ~3; j < hi; j += 4) {
+    float w[C::RT][4];
 #pragma unroll
-    for (int i = 0; i < C::RT; ++i) w[i] = p[i * ldp + j];
+    for (int i = 0; i < C::RT; ++i) {
+      const float4 x = *reinterpret_cast<const float4*>(p + i * ldp + j);
+      w[i][0] = x.x; w[i][1] = x.y; w[i][2] = x.z; w[i][3] = x.w;
+    }
 #pragma unroll
-    for (int m = 0; m < CB; ++m)
-      if (m == 0 || c + 64 * m < dh) {
-        const float4 v = *reinterpret_cast<const float4*>(B + (j - b0) * ldh + c + 64 * m);
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int i = 0; i < C::RT; ++i) {
-          acc[i][m][0] = fmaf(w[i], v.x, acc[i][m][0]);
-          acc[i][m][1] = fmaf(w[i], v.y, acc[i][m][1]);
-          acc[i][m][2] = fmaf(w[i], v.z, acc[i][m][2]);
-          acc[i][m][3] = fmaf(w[i], v.w, acc[i][m][3]);
+      for (int m = 0; m < CB; ++m)
+        if (m == 0 || c + 64 * m < dh) {
+          const float4 v = *reinterpret_cast<const float4*>(B + (j + q - b0) * ldh + c + 64 * m);
+#pragma unroll
+          for (int i = 0; i < C::RT; ++i) {
+            acc[i][m][0] = fmaf(w[i][q], v.x, acc[i][m][0]);
+            acc[i][m][1] = fmaf(w[i][q], v.y, acc[i][m][1]);
+            acc[i][m][2] = fmaf(w[i][q], v.z, acc[i][m][2]);
+            acc[i][m][3] = fmaf(w[i][q], v.w, acc[i][m][3]);
+          }
         }
-      }
   }
 }
 // acc[i] += sum over queries r in [lo, hi) of P[r][row + i] B[r].
@@ -273,17 +281,18 @@ __device__ __forceinline__ int block_end(int r, int L) {
 // gate to bf16 in turn: a last-bit difference here would move every later
 // rounding, the fp32 decay gradient among the results.)  Hence two phases: all
 // of the row's scores, kept in shared memory for up to kKeep key tiles (beyond
-// that they are formed twice), then exponentials, sum and output.
+// that they are formed twice), then exponentials, sum and output.  share: K and V
+// take turns in one buffer, where that makes room for a second CTA on the SM.
 constexpr int kKeep = 4;
 template <class E, int C4, int CB>
 __global__ void __launch_bounds__(kThreads, 2)
-    attn_fwd_simt_kernel(const __grid_constant__ SimtArgs<E> a, int ldp) {
+    attn_fwd_simt_kernel(const __grid_constant__ SimtArgs<E> a, int ldp, int share) {
   pdl_enter();
   using C = Cols<C4, CB>;
   extern __shared__ __align__(16) float sm[];
   const int dh = a.x.dh, ldh = dh + 4;
-  float *Qs = sm, *Ks = Qs + kTile * ldh, *Vs = Ks + kTile * ldh, *Ps = Vs + kTile * ldh,
-        *inv = Ps + kTile * ldp;  // [64]
+  float *Qs = sm, *Ks = Qs + kTile * ldh, *Vs = share ? Ks : Ks + kTile * ldh,
+        *Ps = Vs + kTile * ldh, *inv = Ps + kTile * ldp;  // inv: [64]
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int h = blockIdx.y, b = blockIdx.z;
   const TileAt tt = tile_at(a, blockIdx.x);
@@ -309,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
   };
   fill(Qs, ldh, a.x.Q + (row0 + tt.t0) * a.x.ld + c0, a.x.ld, tt.rows, dh, a.vec);
-  load_tile(Vs, a.x.V, 0);
+  if (!share) load_tile(Vs, a.x.V, 0);
   float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
   for (int kt = 0; kt <= tt.j; ++kt) {
     if (kt > 0) __syncthreads();
@@ -352,11 +361,15 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();  // keep: the probabilities are written; else the last tile is used up
     if (!keep) {
       load_tile(Ks, a.x.K, kt);
-      load_tile(Vs, a.x.V, kt);
+      if (!share) load_tile(Vs, a.x.V, kt);
       __syncthreads();
       exps(kt, 0);
       __syncthreads();
-    } else if (kt > 0) {
+      if (share) {
+        load_tile(Vs, a.x.V, kt);
+        __syncthreads();
+      }
+    } else if (share || kt > 0) {
       load_tile(Vs, a.x.V, kt);
       __syncthreads();
     }
@@ -482,7 +495,7 @@ __device__ __forceinline__ void store_dq(const SimtArgs<E>& a, const TileAt& tt,
 // L > 64, per query tile: Drow_t = dO_t . O_t, and
 // dQ_t = scale * sum_j P_tj (dO_t . v_j - Drow_t) k_j over the block's key tiles.
 template <class E, int C4, int CB>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     attn_bwd_q_simt_kernel(const __grid_constant__ SimtArgs<E> a) {
   pdl_enter();
   extern __shared__ __align__(16) float sm[];
@@ -529,7 +542,7 @@ __global__ void __launch_bounds__(kThreads)
 // tile is its own and only query tile): Drow is formed here and dQ joins, one
 // pass instead of two.
 template <class E, int C4, int CB, bool FUSED>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     attn_bwd_kv_simt_kernel(const __grid_constant__ SimtArgs<E> a) {
   pdl_enter();
   extern __shared__ __align__(16) float sm[];
@@ -626,11 +639,13 @@ int simt_smem(int tiles, int cols, int dh) {
   return kTile * (tiles * (dh + 4) + cols) * (int)sizeof(float);
 }
 
+constexpr int kHalfSm = 113 * 1024;  // shared memory of each of two CTAs on an SM
+
 template <class K, class E, class... X>
 cudaError_t simt_launch(const Launch& lc, K kern, std::atomic<unsigned long long>* opted, int tiles,
                         int cols, int max_cols, const AttnArgs& f, const SimtArgs<E>& a, X... x) {
   // the limit is raised once per kernel and device, to the largest size needed
-  if (cudaError_t e = smem_opt_in(kern, simt_smem(tiles, max_cols, kMaxDh), opted);
+  if (cudaError_t e = smem_opt_in(kern, simt_smem(std::max(tiles, 3), max_cols, kMaxDh), opted);
       e != cudaSuccess)
     return e;
   const int nx = f.L <= kTile ? (f.T + a.rows - 1) / a.rows : (f.T + f.L - 1) / f.L * a.tpb;
@@ -657,8 +672,9 @@ cudaError_t fwd_typed(const Launch& lc, const AttnArgs& f) {
     static std::atomic<unsigned long long> opted{0};
     // the row's scores (four more columns of padding), and one for the sums
     const int ldp = a.tpb <= kKeep ? a.tpb * kTile + 4 : kPld;
+    const int share = simt_smem(3, ldp + 1, f.dh) > kHalfSm && simt_smem(2, ldp + 1, f.dh) <= kHalfSm;
     return simt_launch(lc, attn_fwd_simt_kernel<E, decltype(c4)::value, decltype(cb)::value>,
-                       &opted, 3, ldp + 1, kKeep * kTile + 5, f, a, ldp);
+                       &opted, 3 - share, ldp + 1, kKeep * kTile + 5, f, a, ldp, share);
   });
 }
 
