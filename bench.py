@@ -232,7 +232,7 @@ KERNEL_SOURCES = {
     "attn_fwd_tc": ("attn_tc.cu", "attn_common.cuh"),
     "attn_bwd_tc": ("attn_tc.cu", "attn_common.cuh"),
     "attn_fwd_fl": ("attn_flash.cu", "attn_common.cuh"),
-    "attn_bwd_fl": ("attn_flash.cu", "attn_common.cuh"),
+    "attn_bwd_fl": ("attn_blk.cu", "attn_flash.cu", "attn_common.cuh"),
     "attn_fwd_simt": ("attn_simt.cu",),
     "attn_bwd_simt": ("attn_simt.cu",),
 }

@@ -65,7 +65,9 @@ int bcmt_test_gemm_group(int M0, int N0, int K0, const void* A0, long lda0, cons
  * width 16/32/64, L <= 128), 2 key-tile-walking tcgen05 (head width 16/32/64, L
  * dividing or a multiple of 128; its backward also writes drow), 3 the
  * CUDA-core forward and the tcgen05 backward for any bf16 shape (which writes
- * drow for L > 128).  Returns 0, or -1 on error (bcmt_last_error()). */
+ * drow for L > 128), 4 the one-pass tcgen05 backward of blocks of several
+ * tiles (L = 128 m, 2 <= m <= 8 / 6 / 2 for head width 16 / 32 / 64; also
+ * writes drow).  Returns 0, or -1 on error (bcmt_last_error()). */
 int bcmt_test_attn(int impl, int backward, const bcmt_params* p, const void* q, const void* k,
                    const void* v, long ld, void* o, float* lse, const void* dO, float* drow,
                    void* dq, void* dk, void* dv, long ld_d, void* stream);

@@ -1,0 +1,473 @@
+// Backward of the intra-block causal attention on the tcgen05 tensor cores (Sec.
+// 3.3) for blocks of several 128-token tiles, one pass: head widths DH in {16, 32,
+// 64}, L = 128 m with m <= 8, 6, 2 (what TMEM holds).
+//
+// A CTA takes one (block, head) at a time and walks its pairs (key tile kt, query
+// tile qt >= kt), kt outer, forming S = Q K^T and dP = dO V^T of a pair once for
+// all three gradients:  dV_kt += P^T dO_qt, dK_kt += dS^T Q_qt, dQ_qt += dS K_kt.
+// The block's Q and dO tiles stay in shared memory, K and V are double-buffered;
+// TMEM holds S and dP (128 columns each), dK, dV of the current kt and dQ of every
+// query tile.  dQ_kt is complete with key tile kt, so each kt ends by storing dQ,
+// dK and dV of one tile.  One CTA per SM, persistent, with a warp for each job that
+// would otherwise sit in the elementwise warps' way:
+//   warps 0-7  a pair's S and dP into registers, P and dS to shared memory; a
+//              finished tile's gradients to the buffers that held its operands
+//              (warp w: TMEM lane quarter w % 4, half w / 4 of the key columns);
+//   warp 8     issues the products: the next pair's S and dP as soon as the columns
+//              are free, then the pair's three gradient products;
+//   warp 9     stores finished tiles and loads the next block's into their place, so
+//              a block's first loads run under the last one's work;
+//   warps 10, 11  the next block's row statistics (Drow = dO . O); the first block's
+//              come from warps 0-7.
+//
+// What bounds it: a pair's 26 or more MMAs and their issue (about 1700 cycles at DH =
+// 16) next to the elementwise chain (1400: 64 exponentials a thread, 64 KB of stores),
+// the two overlapping but for the first pair of a block; at DH = 64, also the loads.
+// Per pair 1.5 us at DH = 16, 4.2 us at DH = 64 (L 256, HBM's share 1.9 us).  The
+// two-kernel form (attn_flash.cu, which keeps the shapes that do not fit) forms S and
+// dP once for dQ and once more for dK, dV, and is the slower one from the smallest
+// grid on: in us, two kernels -> this, for 8 / 152 / 608 (block, head)s:
+//   DH 16, L 256    23 -> 15    27 -> 15    64 -> 34
+//   DH 16, L 1024   64 -> 62   148 -> 64   470 -> 218
+//   DH 32, L 512    42 -> 27    74 -> 31   206 -> 83
+//   DH 64, L 256    25 -> 19    36 -> 25   115 -> 56
+#include "attn_common.cuh"
+#include "common.cuh"
+#include "internal.h"
+#include "tc.cuh"
+#include "tmap.h"
+
+namespace bcmt {
+using namespace attn;
+
+namespace {
+constexpr int kTile = 128;
+constexpr int kWorkers = 256;
+constexpr int kMmaWarp = 8, kIoWarp = 9, kStatWarp = 10;
+constexpr int kStatThreads = 64;
+constexpr int kThreads = 384;
+constexpr int kMaxM = 8;
+
+struct BlkArgs {
+  const bf16 *O, *dO;
+  long ld_o;
+  const float* lse;
+  float* Drow;
+  int T, H, L, m;
+  int nb, total;  // blocks a sequence, (block, head, batch) items
+  float scale;
+  unsigned* status;
+};
+
+// P and dS (32 KB each), m tiles of Q and of dO, two of K and of V, two blocks' row
+// statistics, barriers.
+template <int DH> constexpr int blk_smem(int m) {
+  return 1024 + 65536 + (2 * m + 4) * (int)Geo<DH>::tile + 2 * m * kTile * 8 + 256;
+}
+
+// Item it: heads of one block are neighbours (their rows share memory pages).
+struct Item {
+  int t0, h, b, nq;
+  __device__ Item(const BlkArgs& a, int it) {
+    const int x = it / a.H;
+    h = it - x * a.H;
+    b = x / a.nb;
+    t0 = (x - b * a.nb) * a.L;
+    nq = (min(a.L, a.T - t0) + kTile - 1) / kTile;
+  }
+};
+
+// The bf16 tile row r as a TMA store takes it.
+template <int DH>
+__device__ __forceinline__ void blk_stage(uint8_t* tile, int r, const float* v) {
+#pragma unroll
+  for (int u = 0; u < DH / 8; ++u)
+    *reinterpret_cast<uint4*>(tile + Geo<DH>::unit(r, u)) = pack8(v + 8 * u);
+}
+}  // namespace
+
+template <int DH>
+__global__ void __launch_bounds__(kThreads, 1)
+    attn_bwd_blk_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
+                        const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO,
+                        const __grid_constant__ CUtensorMap mdQ, const __grid_constant__ CUtensorMap mdK,
+                        const __grid_constant__ CUtensorMap mdV, const __grid_constant__ BlkArgs a) {
+  using G = Geo<DH>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align1024(smem_raw);
+  uint8_t* sP = smem;
+  uint8_t* sS = smem + 32768;
+  uint8_t* sQ = smem + 65536;            // m tiles; a finished dQ tile is staged in its own
+  uint8_t* sdO = sQ + a.m * G::tile;     // m tiles; dV likewise
+  uint8_t* sK = sdO + a.m * G::tile;     // two; dK likewise
+  uint8_t* sV = sK + 2 * G::tile;        // two
+  float2* stat = reinterpret_cast<float2*>(sV + 2 * G::tile);  // [2][m * 128]: -lse log2 e, -Drow scale
+  // Barriers in pairs are used in turn; c counts a CTA's key tiles, p its pairs and
+  // n its items, over all items.
+  uint64_t* bar_q = reinterpret_cast<uint64_t*>(stat + 2 * a.m * kTile);  // [8] Q, dO tile loaded
+  uint64_t* bar_k = bar_q + kMaxM;  // [2] K, V of key tile c loaded
+  uint64_t* bar_e = bar_k + 2;      // [2] gradients of key tile c staged (8 warps)
+  uint64_t* bar_t = bar_e + 2;      // [2] row statistics of item n written (2 warps)
+  uint64_t* bar_d = bar_t + 2;      // [2] row statistics of item n read (8 warps)
+  uint64_t* bar_s = bar_d + 2;      // S, dP of pair p
+  uint64_t* bar_g = bar_s + 1;      // gradient products of pair p
+  uint64_t* bar_r = bar_g + 1;      // S and dP of pair p in registers (8 warps)
+  uint64_t* bar_p = bar_r + 1;      // P and dS of pair p in shared memory (8 warps)
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar_p + 1);
+  constexpr uint32_t kDK = 256, kDV = kDK + DH, kDQ = kDV + DH;
+
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const int step = gridDim.x;
+
+  if (warp == 0 && tc::elect_one()) {
+    for (int i = 0; i < kMaxM; ++i) tc::mbar_init(&bar_q[i], 1);
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&bar_k[i], 1);
+      tc::mbar_init(&bar_e[i], kWorkers / 32);
+      tc::mbar_init(&bar_t[i], kStatThreads / 32);
+      tc::mbar_init(&bar_d[i], kWorkers / 32);
+    }
+    tc::mbar_init(bar_s, 1);
+    tc::mbar_init(bar_g, 1);
+    tc::mbar_init(bar_r, kWorkers / 32);
+    tc::mbar_init(bar_p, kWorkers / 32);
+    tc::fence_mbar_init();
+  }
+  if (warp == kMmaWarp) {
+    tc::tmem_alloc(tslot, 512);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot;
+  pdl_enter();
+  bool ok = true;
+  // Statistics of an item's rows by n threads: Drow = dO . O, and what P and dS take.
+  auto row_stats = [&](const Item& j, float2* dst, int i, int n) {
+    const bf16 *O = after_wait(a.O), *dO = after_wait(a.dO);
+    const float* lse = after_wait(a.lse);
+    for (; i < j.nq * kTile; i += n) {
+      float2 st = make_float2(0.f, 0.f);
+      if (j.t0 + i < a.T) {
+        const long row = (long)j.b * a.T + j.t0 + i, o = row * a.ld_o + j.h * DH;
+        const long li = ((long)j.b * a.H + j.h) * a.T + j.t0 + i;
+        float d = 0.f;
+#pragma unroll
+        for (int u = 0; u < DH / 8; ++u) {
+          float ov[8], gv[8];
+          load8(O + o + 8 * u, ov);
+          load8(dO + o + 8 * u, gv);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) d = fmaf(ov[e], gv[e], d);
+        }
+        a.Drow[li] = d;
+        st = make_float2(-lse[li] * kLog2e, -d * a.scale);
+      }
+      dst[i] = st;
+    }
+  };
+
+  if (warp == kMmaWarp) {
+    // ------------------------------------------------------------ products
+    constexpr uint32_t idS = tc::idesc_bf16(128, 128, 0, 0), idMN = tc::idesc_bf16(128, DH, 1, 1),
+                       idKM = tc::idesc_bf16(128, DH, 0, 1);
+    // operand descriptors of the buffers' starts; a step along one adds its bytes / 16
+    const uint64_t kq = G::kmaj(sQ, 0, 0), kg = G::kmaj(sdO, 0, 0), kk0 = G::kmaj(sK, 0, 0),
+                   kv = G::kmaj(sV, 0, 0), nq0 = G::mnmaj(sQ, 0, 0), ng = G::mnmaj(sdO, 0, 0),
+                   nk = G::mnmaj(sK, 0, 0), ap = tc::sdesc(tc::smem_u32(sP), 16384, 1024),
+                   as = tc::sdesc(tc::smem_u32(sS), 16384, 1024), ks = p_kmaj(sS, 0, 0);
+    constexpr uint32_t kT = G::tile / 16, kN = G::span;  // a tile; 16 rows of one
+    uint32_t qph = 0;  // parity of each Q, dO slot's next load
+    // S and dP of pair (kt, qt), whose key tile is the CTA's c-th, into columns 0 .. 255
+    auto issue_s = [&](int c, int kt, int qt) {
+      if (qt == kt) ok = ok && tc::mbar_wait(&bar_k[c & 1], (c >> 1) & 1, a.status);
+      if (kt == 0) {
+        ok = ok && tc::mbar_wait(&bar_q[qt], (qph >> qt) & 1, a.status);
+        qph ^= 1u << qt;
+      }
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        if (ok) {
+          const uint64_t q0 = kq + qt * kT, g0 = kg + qt * kT, k0 = kk0 + (c & 1) * kT,
+                         v0 = kv + (c & 1) * kT;
+#pragma unroll
+          for (int kk = 0; kk < DH / 16; ++kk)
+            tc::mma_bf16(tmem, q0 + kk * 2, k0 + kk * 2, idS, kk > 0 ? 1u : 0u);
+#pragma unroll
+          for (int kk = 0; kk < DH / 16; ++kk)
+            tc::mma_bf16(tmem + 128, g0 + kk * 2, v0 + kk * 2, idS, kk > 0 ? 1u : 0u);
+        }
+        tc::mma_commit(bar_s);
+      }
+      __syncwarp();
+    };
+    issue_s(0, 0, 0);
+    int p = 0, c = 0;
+    for (int it = blockIdx.x; it < a.total; it += step) {
+      const int nq = Item(a, it).nq;
+      for (int kt = 0; kt < nq; ++kt, ++c)
+        for (int qt = kt; qt < nq; ++qt, ++p) {
+          ok = ok && tc::mbar_wait(bar_r, p & 1, a.status);
+          if (qt + 1 < nq)
+            issue_s(c, kt, qt + 1);
+          else if (kt + 1 < nq)
+            issue_s(c + 1, kt + 1, kt + 1);
+          ok = ok && tc::mbar_wait(bar_p, p & 1, a.status);
+          tc::fence_after_sync();
+          if (tc::elect_one()) {
+            if (ok) {
+              const uint64_t q0 = nq0 + qt * kT, g0 = ng + qt * kT, k0 = nk + (c & 1) * kT;
+              const uint32_t dq = tmem + kDQ + (uint32_t)(qt * DH);
+              const uint32_t first = qt == kt ? 0u : 1u, firstq = kt == 0 ? 0u : 1u;
+#pragma unroll
+              for (int kk = 0; kk < kTile / 16; ++kk)  // dV += P^T dO
+                tc::mma_bf16(tmem + kDV, ap + kk * 128, g0 + kk * kN, idMN, kk > 0 ? 1u : first);
+#pragma unroll
+              for (int kk = 0; kk < kTile / 16; ++kk)  // dK += dS^T Q
+                tc::mma_bf16(tmem + kDK, as + kk * 128, q0 + kk * kN, idMN, kk > 0 ? 1u : first);
+#pragma unroll
+              for (int kk = 0; kk < kTile / 16; ++kk)  // dQ += dS K
+                tc::mma_bf16(dq, ks + (kk >> 2) * 1024 + (kk & 3) * 2, k0 + kk * kN, idKM,
+                             kk > 0 ? 1u : firstq);
+            }
+            tc::mma_commit(bar_g);
+          }
+          __syncwarp();
+          // the next block's first tiles may come in only after these products
+          if (kt + 1 == nq && it + step < a.total) issue_s(c + 1, 0, 0);
+        }
+    }
+  } else if (warp == kIoWarp) {
+    // ------------------------------------------------------ loads and stores
+    if (tc::elect_one()) {
+      auto load_kv = [&](const Item& i, int kt, int c) {
+        tc::mbar_arrive_expect_tx(&bar_k[c & 1], 2 * G::tile);
+        tc::tma_load_3d(sK + (c & 1) * G::tile, &mK, &bar_k[c & 1], i.h * DH, i.t0 + kt * kTile, i.b);
+        tc::tma_load_3d(sV + (c & 1) * G::tile, &mV, &bar_k[c & 1], i.h * DH, i.t0 + kt * kTile, i.b);
+      };
+      auto load_q = [&](const Item& i, int qt) {
+        tc::mbar_arrive_expect_tx(&bar_q[qt], 2 * G::tile);
+        tc::tma_load_3d(sQ + qt * G::tile, &mQ, &bar_q[qt], i.h * DH, i.t0 + qt * kTile, i.b);
+        tc::tma_load_3d(sdO + qt * G::tile, &mdO, &bar_q[qt], i.h * DH, i.t0 + qt * kTile, i.b);
+      };
+      int kit = blockIdx.x, kkt = 0, kc = 0;  // the next key tile to load
+      auto next_kv = [&]() {
+        if (kit >= a.total) return;
+        const Item i(a, kit);
+        load_kv(i, kkt, kc++);
+        if (++kkt == i.nq) kkt = 0, kit += step;
+      };
+      next_kv();
+      {
+        const Item i(a, blockIdx.x);
+        load_q(i, 0);
+        next_kv();
+        for (int qt = 1; qt < i.nq; ++qt) load_q(i, qt);
+      }
+      int c = 0;
+      for (int it = blockIdx.x; it < a.total; it += step) {
+        const Item i(a, it);
+        const bool more = it + step < a.total;
+        const Item j(a, more ? it + step : it);
+        for (int kt = 0; kt < i.nq; ++kt, ++c) {
+          ok = ok && tc::mbar_wait(&bar_e[c & 1], (c >> 1) & 1, a.status);
+          if (ok) {
+            const int x = i.h * DH, t = i.t0 + kt * kTile;
+            tc::tma_store_3d(&mdQ, sQ + kt * G::tile, x, t, i.b);
+            tc::tma_store_3d(&mdK, sK + (c & 1) * G::tile, x, t, i.b);
+            tc::tma_store_3d(&mdV, sdO + kt * G::tile, x, t, i.b);
+            tc::tma_store_commit();
+            tc::tma_store_wait_read<0>();  // the staging is read: its buffers are free
+            next_kv();
+            if (more && kt < j.nq) load_q(j, kt);
+            if (more && kt + 1 == i.nq)
+              for (int qt = i.nq; qt < j.nq; ++qt) load_q(j, qt);
+          }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp >= kStatWarp) {
+    // ------------------------------------------------ the next items' statistics
+    int n = 0;
+    for (int it = blockIdx.x; it < a.total; it += step, ++n) {
+      if (n >= 2) ok = ok && tc::mbar_wait(&bar_d[n & 1], ((n >> 1) - 1) & 1, a.status);
+      if (n > 0) row_stats(Item(a, it), stat + (n & 1) * a.m * kTile, tid - kStatWarp * 32, kStatThreads);
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bar_t[n & 1]);
+    }
+  } else {
+    // ------------------------------------------------- elementwise, results
+    const int q = warp & 3, hf = warp >> 2;
+    const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+    const int r = q * 32 + lane;
+    const float sl2 = a.scale * kLog2e;
+    const float2 sl2x2 = make_float2(sl2, sl2), sc2 = make_float2(a.scale, a.scale);
+    int p = 0, c = 0, n = 0;
+    for (int it = blockIdx.x; it < a.total; it += step, ++n) {
+      const int nq = Item(a, it).nq;
+      const float2* rs = stat + (n & 1) * a.m * kTile + r;
+      if (n == 0) {  // nothing to run under yet: all eight warps
+        row_stats(Item(a, it), stat, tid, kWorkers);
+        tc::bar_sync(1, kWorkers);
+      }
+      ok = ok && tc::mbar_wait(&bar_t[n & 1], (n >> 1) & 1, a.status);
+      for (int kt = 0; kt < nq; ++kt, ++c) {
+        for (int qt = kt; qt < nq; ++qt, ++p) {
+          const bool diag = qt == kt;
+          const float2 st = rs[qt * kTile];
+          ok = ok && tc::mbar_wait(bar_s, p & 1, a.status);
+          tc::fence_after_sync();
+          uint32_t s[2][32], dp[2][32];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            tc::tmem_ld32_issue(trow + (uint32_t)(hf * 64 + c * 32), s[c]);
+            tc::tmem_ld32_issue(trow + 128u + (uint32_t)(hf * 64 + c * 32), dp[c]);
+          }
+          tc::tmem_wait();
+          tc::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(bar_r);  // the columns are free
+          // P = 2^(s scale log2 e - lse log2 e), dS = P (dP scale - Drow scale): packed
+          // bf16 pairs in place of the loaded words; keys past the row are 0 (diagonal)
+          const float2 nl2 = make_float2(st.x, st.x), nd2 = make_float2(st.y, st.y);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int ch = 2 * hf + c;  // the warp's rows end in chunk q of the diagonal pair
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+              const float2 e = __ffma2_rn(
+                  make_float2(__uint_as_float(s[c][j]), __uint_as_float(s[c][j + 1])), sl2x2, nl2);
+              const float2 d = __ffma2_rn(
+                  make_float2(__uint_as_float(dp[c][j]), __uint_as_float(dp[c][j + 1])), sc2, nd2);
+              const float x = ex2(e.x), y = ex2(e.y);
+              s[c][j >> 1] = pack2(x, y);
+              dp[c][j >> 1] = pack2(x * d.x, y * d.y);
+            }
+            if (diag && ch >= q) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const int k = 32 * ch + 2 * j;
+                const uint32_t keep = (k <= r ? 0xffffu : 0u) | (k < r ? 0xffff0000u : 0u);
+                s[c][j] &= keep;
+                dp[c][j] &= keep;
+              }
+            }
+          }
+          // the last pair's products have read P and dS
+          if (p > 0) ok = ok && tc::mbar_wait(bar_g, (p - 1) & 1, a.status);
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              put_unit(sP, r, hf * 8 + c * 4 + u,
+                       make_uint4(s[c][4 * u], s[c][4 * u + 1], s[c][4 * u + 2], s[c][4 * u + 3]));
+              put_unit(sS, r, hf * 8 + c * 4 + u,
+                       make_uint4(dp[c][4 * u], dp[c][4 * u + 1], dp[c][4 * u + 2], dp[c][4 * u + 3]));
+            }
+          tc::fence_proxy_async_smem();
+          tc::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(bar_p);
+        }
+        // ---- key tile kt is done: its dK and dV, and dQ of query tile kt
+        ok = ok && tc::mbar_wait(bar_g, (p - 1) & 1, a.status);
+        tc::fence_after_sync();
+        {
+          float v[DH];
+          if (hf == 0) {
+            tmem_row<DH>(trow + kDV, v);
+            blk_stage<DH>(sdO + kt * G::tile, r, v);
+            tmem_row<DH>(trow + kDQ + (uint32_t)(kt * DH), v);
+            blk_stage<DH>(sQ + kt * G::tile, r, v);
+          } else {
+            tmem_row<DH>(trow + kDK, v);
+            blk_stage<DH>(sK + (c & 1) * G::tile, r, v);
+          }
+        }
+        tc::fence_proxy_async_smem();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) {
+          tc::mbar_arrive(&bar_e[c & 1]);
+          if (kt + 1 == nq) tc::mbar_arrive(&bar_d[n & 1]);
+        }
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == kMmaWarp) tc::tmem_dealloc(tmem, 512);
+}
+
+// ========================================================================= host
+// TMEM: S, dP (256 columns), dK, dV, and dQ of each of the block's tiles.
+bool attn_blk_supported(int dh, int L) {
+  const int m = L / kTile;
+  return L % kTile == 0 && m >= 2 && m <= kMaxM && 256 + (2 + m) * dh <= 512;
+}
+
+namespace {
+template <int DH>
+bool blk_map(CUtensorMap* m, const void* base, long ld, int D, int T, int B) {
+  const uint64_t dims[3] = {(uint64_t)D, (uint64_t)T, (uint64_t)B};
+  const uint64_t st[2] = {(uint64_t)ld * 2, (uint64_t)ld * 2 * (uint64_t)T};
+  const uint32_t box[3] = {DH, kTile, 1};
+  const CUtensorMapSwizzle sw = DH == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : DH == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                           : CU_TENSOR_MAP_SWIZZLE_32B;
+  return make_tmap_bf16(m, base, 3, dims, st, box, sw);
+}
+
+template <int DH>
+cudaError_t bwd_blk(const Launch& lc, const AttnBwdArgs& ab) {
+  const AttnArgs& f = ab.f;
+  const int D = f.H * DH;
+  CUtensorMap m[7];
+  if (!blk_map<DH>(&m[0], f.Q, f.ld_qkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[1], f.K, f.ld_qkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[2], f.V, f.ld_qkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[3], ab.dO, f.ld_o, D, f.T, f.B) ||
+      !blk_map<DH>(&m[4], ab.dQ, ab.ld_dqkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[5], ab.dK, ab.ld_dqkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[6], ab.dV, ab.ld_dqkv, D, f.T, f.B))
+    return cudaErrorInvalidValue;
+  BlkArgs a;
+  a.O = (const bf16*)f.O;
+  a.dO = (const bf16*)ab.dO;
+  a.ld_o = f.ld_o;
+  a.lse = f.lse;
+  a.Drow = ab.Drow;
+  a.T = f.T;
+  a.H = f.H;
+  a.L = f.L;
+  a.m = f.L / kTile;
+  a.nb = (f.T + f.L - 1) / f.L;
+  const long total = (long)a.nb * f.H * f.B;
+  if (total > INT_MAX / 2) return cudaErrorNotSupported;
+  a.total = (int)total;
+  a.scale = 1.0f / sqrtf((float)DH);
+  a.status = lc.status;
+  auto kern = attn_bwd_blk_kernel<DH>;
+  constexpr int most = blk_smem<DH>(DH == 64 ? 2 : DH == 32 ? 6 : kMaxM);
+  static std::atomic<unsigned long long> opted{0};
+  if (cudaError_t e = smem_opt_in(kern, most, &opted); e != cudaSuccess) return e;
+  cudaError_t e = launch_k(kern, dim3(a.total < sm_count() ? a.total : sm_count()), dim3(kThreads),
+                           blk_smem<DH>(a.m), lc.stream, m[0], m[1], m[2], m[3], m[4], m[5], m[6],
+                           a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t attn_bwd_blk(const Launch& lc, const AttnBwdArgs& a) {
+  if (!attn_blk_supported(a.f.dh, a.f.L)) return cudaErrorNotSupported;
+  switch (a.f.dh) {
+    case 16: return bwd_blk<16>(lc, a);
+    case 32: return bwd_blk<32>(lc, a);
+    case 64: return bwd_blk<64>(lc, a);
+    default: return cudaErrorNotSupported;
+  }
+}
+
+}  // namespace bcmt

@@ -18,7 +18,9 @@
 //    registers; O and the log-sum-exp are stored at the end.  At L > 128
 //    the layer runs the half-tile form (64-key halves, 128 TMEM columns per
 //    CTA, more CTAs per SM).
-//  * backward, two kernels (no atomics, fixed summation order):
+//  * backward, for the shapes that attn_blk.cu's one pass does not fit (DH = 32 with
+//    L >= 896, DH = 64 with L >= 384), two kernels (no atomics, fixed summation
+//    order):
 //      dQ:  per query tile, Drow = dO . O, then per key tile and 64-key half
 //           S, dP (N = 64), dS = P (dP - Drow) scale, dQ += dS K (TMEM);
 //      dKV: per key tile, per query tile and 64-query half S^T = K Q^T,

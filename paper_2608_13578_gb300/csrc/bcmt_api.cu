@@ -1013,7 +1013,8 @@ bcmt_status bcmt_backward(const bcmt_params* p, const void* dy, const void* x_or
       e = attn_bwd_tc(lc, ab);
     } else if (attn_kind(g) == 2) {
       pr.begin("attn_bwd_fl");
-      e = attn_bwd_fl(lc, ab);
+      // one pass where its accumulators fit: faster at every grid size (attn_blk.cu)
+      e = attn_blk_supported(g.dh, g.L) ? attn_bwd_blk(lc, ab) : attn_bwd_fl(lc, ab);
     } else if (attn_kind(g) == 3) {
       pr.begin("attn_bwd_gen");
       e = attn_bwd_gen(lc, ab);
@@ -1331,6 +1332,7 @@ int bcmt_test_attn(int impl, int backward, const bcmt_params* p, const void* q, 
     e = impl == 1 ? attn_bwd_tc(lc, ab)
         : impl == 2 ? attn_bwd_fl(lc, ab)
         : impl == 3 ? attn_bwd_gen(lc, ab)
+        : impl == 4 ? attn_bwd_blk(lc, ab)
                     : attn_bwd_simt(lc, g.dtype, ab);
   }
   if (e != cudaSuccess) {

@@ -250,6 +250,8 @@ struct TcCfg {
   static constexpr int TMEM_COLS = 2 * BN;  // two accumulators
 };
 
+}  // namespace
+
 int sm_count() {
   static int n = 0;
   if (!n) {
@@ -260,6 +262,8 @@ int sm_count() {
   }
   return n;
 }
+
+namespace {
 }  // namespace
 
 // Persistent, warp-specialised tcgen05 GEMM.  Tiles are 128 x BN output

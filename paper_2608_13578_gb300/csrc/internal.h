@@ -196,6 +196,13 @@ bool attn_tc_supported(int dtype, int dh, int L);
 bool attn_fl_supported(int dtype, int dh, int L);
 cudaError_t attn_fwd_fl(const Launch& lc, const AttnArgs& a);
 cudaError_t attn_bwd_fl(const Launch& lc, const AttnBwdArgs& a);
+int sm_count();  // SMs of the current device (of the first one asked about)
+
+// The backward of blocks of several tiles in one pass (also writes Drow), where its
+// accumulators fit TMEM.
+bool attn_blk_supported(int dh, int L);
+cudaError_t attn_bwd_blk(const Launch& lc, const AttnBwdArgs& a);
+
 // tcgen05 attention backward for every other bf16 shape: head widths that are
 // multiples of 8 up to 128, any L up to 1024 (P and dS as two bf16 parts each).
 bool attn_gen_supported(int dtype, int dh, int L);
