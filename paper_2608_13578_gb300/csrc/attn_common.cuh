@@ -44,11 +44,11 @@ struct Geo {
   static constexpr uint32_t layout = DH == 64 ? 2u : DH == 32 ? 4u : 6u;
   // K-major [rows x DH] operand at row offset `row0`, K step kk (16 columns)
   static __device__ __forceinline__ uint64_t kmaj(const uint8_t* t, int row0, int kk) {
-    return tc::sdesc_sw(tc::smem_u32(t) + row0 * span + kk * 32, 16, sbo, layout);
+    return tc::desc_at(tc::sdesc_sw(tc::smem_u32(t), 16, sbo, layout), row0 * span + kk * 32);
   }
   // the same tile read MN-major (DH contiguous = N), K = rows from row0, step kk
   static __device__ __forceinline__ uint64_t mnmaj(const uint8_t* t, int row0, int kk) {
-    return tc::sdesc_sw(tc::smem_u32(t) + (row0 + kk * 16) * span, tile, sbo, layout);
+    return tc::desc_at(tc::sdesc_sw(tc::smem_u32(t), tile, sbo, layout), (row0 + kk * 16) * span);
   }
   // byte offset of 16-byte unit u (columns 8u .. 8u+7) of row r: the unit
   // index is XORed with address bits 7.. of the unswizzled offset (1, 2 or 3
@@ -64,7 +64,8 @@ struct Geo {
 // layout), read K-major from column 64*half, K step kk.  A single 64-column
 // half buffer is read with half = 0 and kk < 4.
 __device__ __forceinline__ uint64_t p_kmaj(const uint8_t* p, int half, int kk) {
-  return tc::sdesc(tc::smem_u32(p) + half * 16384 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
+  return tc::desc_at(tc::sdesc(tc::smem_u32(p), 16, 1024),
+                     half * 16384 + (kk >> 2) * 16384 + (kk & 3) * 32);
 }
 
 // Loads TMEM columns col .. col+DH-1 of the warp's lane quarter (thread = row).

@@ -85,12 +85,13 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
   uint64_t* bar_o = bar + 4;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 5);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   int kstart, nkt;
   key_walk(t0, L, kstart, nkt);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 5; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
     tc::prefetch_tmap(&mV);
   }
   pdl_enter();
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar_k[0], 2 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar_k[0], h * DH, t0, b);
     tc::tma_load_3d(sK0, &mK, &bar_k[0], h * DH, kstart, b);
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
   constexpr uint32_t idS = tc::idesc_bf16(128, 128, 0, 0);
   constexpr uint32_t idO = tc::idesc_bf16(128, DH, 0, 1);
 
-  if (tid == 0) {  // S of the first key tile
+  if (warp0 && tc::elect_one()) {  // S of the first key tile
     const bool okk = tc::mbar_wait(&bar_k[0], 0, status);
     tc::fence_after_sync();
     if (okk) {
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
     tc::tmem_wait();
     tc::fence_before_sync();
     __syncthreads();  // every thread has its scores: the S columns are free
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (kt + 1 < nkt) {  // next tile's scores, under this tile's softmax
         const int nb = (kt + 1) & 1;
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
     tc::fence_before_sync();
     __syncthreads();
 
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       const bool okv = tc::mbar_wait(bar_v, kt & 1, status);
       tc::fence_after_sync();
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(128, NCH <= 2 ? 3 : 2)
     ok = tc::mbar_wait(bar_o, kt & 1, status) && ok;
     tc::fence_after_sync();
     // V and P are free: fetch the next tile's V while this P V is folded in
-    if (tid == 0 && kt + 1 < nkt) {
+    if (warp0 && tc::elect_one() && kt + 1 < nkt) {
       tc::mbar_arrive_expect_tx(bar_v, G::tile);
       tc::tma_load_3d(sV, &mV, bar_v, h * DH, kstart + (kt + 1) * kTile, b);
     }
@@ -350,12 +351,13 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
   uint64_t* bar_o = bar + 4;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 5);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   int kstart, nkt;
   key_walk(t0, L, kstart, nkt);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 5; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     tc::prefetch_tmap(&mV);
   }
   pdl_enter();
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar_k[0], 2 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar_k[0], h * DH, t0, b);
     tc::tma_load_3d(sK0, &mK, &bar_k[0], h * DH, kstart, b);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     tc::mma_commit(bar_s);
   };
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     const bool okk = tc::mbar_wait(&bar_k[0], 0, status);
     tc::fence_after_sync();
     if (okk) issue_s(0, 0);
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     const bool diag = kt == nkt - 1;
     const int kb = NKB == 2 ? (kt & 1) : 0;
     if constexpr (NKB == 1) {
-      if (kt > 0 && tid == 0) {  // this tile's K (loaded during the last tile)
+      if (warp0 && tc::elect_one() && kt > 0) {  // this tile's K (loaded during the last tile)
         const bool okk = tc::mbar_wait(&bar_k[0], kt & 1, status);
         tc::fence_after_sync();
         if (okk && ok) issue_s(0, 0);
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
       tc::tmem_wait();
       tc::fence_before_sync();
       __syncthreads();  // every thread has this half's scores: the S columns are free
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         if (hh == 0) {  // the tile's second half
           if (ok) issue_s(kb, 1);
@@ -499,7 +501,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
       tc::fence_before_sync();
       __syncthreads();
 
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         const bool okv = tc::mbar_wait(bar_v, kt & 1, status);
         tc::fence_after_sync();
@@ -517,7 +519,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
       tc::fence_after_sync();
       // V is free after the tile's second P V: fetch the next tile's V while
       // this product is folded in
-      if (tid == 0 && hh == 1 && kt + 1 < nkt) {
+      if (warp0 && tc::elect_one() && hh == 1 && kt + 1 < nkt) {
         tc::mbar_arrive_expect_tx(bar_v, G::tile);
         tc::tma_load_3d(sV, &mV, bar_v, h * DH, kstart + (kt + 1) * kTile, b);
       }
@@ -559,12 +561,13 @@ __global__ void __launch_bounds__(128)
   uint64_t* bar = reinterpret_cast<uint64_t*>(sV + G::tile);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   int kstart, nkt;
   key_walk(t0, L, kstart, nkt);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -576,7 +579,7 @@ __global__ void __launch_bounds__(128)
   O = after_wait(O);
   dO = after_wait(dO);
   lse = after_wait(lse);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
     tc::tma_load_3d(sdO, &mdO, &bar[0], h * DH, t0, b);
@@ -632,7 +635,7 @@ __global__ void __launch_bounds__(128)
     }
     tc::mma_commit(&bar[1]);
   };
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     ok = tc::mbar_wait(&bar[0], 0, status) && ok;
     tc::fence_after_sync();
     issue_sdp(0);
@@ -657,7 +660,7 @@ __global__ void __launch_bounds__(128)
       tc::tmem_wait();
       tc::fence_before_sync();
       __syncthreads();  // every thread has this half's S and dP: the columns are free
-      if (tid == 0 && hh == 0) {
+      if (warp0 && tc::elect_one() && hh == 0) {
         tc::fence_after_sync();
         issue_sdp(1);
       }
@@ -692,7 +695,7 @@ __global__ void __launch_bounds__(128)
       tc::fence_proxy_async_smem();
       tc::fence_before_sync();
       __syncthreads();
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         if (ok) {
           constexpr uint32_t idQ = tc::idesc_bf16(128, DH, 0, 1);
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(128)
     }
     // the next key tile may overwrite K and V once this tile's products are
     // done (the half-1 commit covers every earlier product); then its half 0
-    if (tid == 0 && kt + 1 < nkt) {
+    if (warp0 && tc::elect_one() && kt + 1 < nkt) {
       ok = tc::mbar_wait(&bar[3], kt & 1, status) && ok;
       tc::mbar_arrive_expect_tx(&bar[0], 2 * G::tile);
       tc::tma_load_3d(sK, &mK, &bar[0], h * DH, kstart + (kt + 1) * kTile, b);
@@ -758,12 +761,13 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
   uint64_t* bar = reinterpret_cast<uint64_t*>(sV + G::tile);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 6);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   int kstart, nkt;
   key_walk(t0, L, kstart, nkt);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 6; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -775,7 +779,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
   O = after_wait(O);
   dO = after_wait(dO);
   lse = after_wait(lse);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
     tc::tma_load_3d(sdO, &mdO, &bar[0], h * DH, t0, b);
@@ -832,7 +836,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     }
     tc::mma_commit(&bar[1]);
   };
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     ok = tc::mbar_wait(&bar[0], 0, status) && ok;
     tc::fence_after_sync();
     issue_sdp(0);
@@ -852,7 +856,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
       tc::tmem_wait();
       tc::fence_before_sync();
       __syncthreads();  // every thread has this quarter's S and dP: the columns are free
-      if (tid == 0 && q < 3) {
+      if (warp0 && tc::elect_one() && q < 3) {
         tc::fence_after_sync();
         issue_sdp(q + 1);
       }
@@ -884,7 +888,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
       tc::fence_proxy_async_smem();
       tc::fence_before_sync();
       __syncthreads();
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         if (ok) {
           constexpr uint32_t idQ = tc::idesc_bf16(128, DH, 0, 1);
@@ -899,7 +903,7 @@ __global__ void __launch_bounds__(128, DH <= 16 ? 4 : 3)
     // the next key tile may overwrite K and V once this tile's products are
     // done (the last quarter's commit covers every earlier product); then its
     // first quarter
-    if (tid == 0 && kt + 1 < nkt) {
+    if (warp0 && tc::elect_one() && kt + 1 < nkt) {
       ok = tc::mbar_wait(&bar[5], kt & 1, status) && ok;
       tc::mbar_arrive_expect_tx(&bar[0], 2 * G::tile);
       tc::tma_load_3d(sK, &mK, &bar[0], h * DH, kstart + (kt + 1) * kTile, b);
@@ -942,14 +946,15 @@ __global__ void __launch_bounds__(128)
   uint64_t* bar = reinterpret_cast<uint64_t*>(sdr + kTile);  // kv, s, q
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 3);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int k0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   // queries that see this key tile: to the end of its block (L >= 128) or of
   // the tile itself (L < 128, block-diagonal mask)
   const int qend = min(L >= kTile ? (k0 / L + 1) * L : k0 + kTile, Tlen);
   const int nqt = (qend - k0 + kTile - 1) / kTile;
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 3; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -960,7 +965,7 @@ __global__ void __launch_bounds__(128)
   pdl_enter();
   lse = after_wait(lse);
   Drow = after_wait(Drow);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, k0, b);
     tc::tma_load_3d(sV, &mV, &bar[0], h * DH, k0, b);
@@ -995,7 +1000,7 @@ __global__ void __launch_bounds__(128)
       slse[tid] = tq < Tlen ? -lse[li] * kLog2e : 0.f;
       sdr[tid] = tq < Tlen ? -Drow[li] * scale : 0.f;
     }
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       ok = tc::mbar_wait(&bar[0], qt & 1, status) && ok;
       tc::fence_after_sync();
     }
@@ -1016,7 +1021,7 @@ __global__ void __launch_bounds__(128)
     };
     for (int hh = 0; hh < 2; ++hh) {
       // half 1's products were issued with half 0's dV/dK (below), ahead of them
-      if (tid == 0 && hh == 0) issue_scores(0);
+      if (warp0 && tc::elect_one() && hh == 0) issue_scores(0);
       __syncwarp();
       ok = tc::mbar_wait(&bar[1], ns & 1, status) && ok;
       ++ns;
@@ -1062,7 +1067,7 @@ __global__ void __launch_bounds__(128)
       tc::fence_proxy_async_smem();
       tc::fence_before_sync();
       __syncthreads();
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         // every thread has read this half's scores out of TMEM (the barrier
         // above): the next half's products go first, under this half's dV/dK
@@ -1084,7 +1089,7 @@ __global__ void __launch_bounds__(128)
       }
       ++nq;
     }
-    if (tid == 0 && qt + 1 < nqt) {
+    if (warp0 && tc::elect_one() && qt + 1 < nqt) {
       ok = tc::mbar_wait(&bar[2], (nq - 1) & 1, status) && ok;
       tc::mbar_arrive_expect_tx(&bar[0], 2 * G::tile);
       tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, q0 + kTile, b);
@@ -1135,12 +1140,13 @@ __global__ void __launch_bounds__(128, 3)
   uint64_t* bar = reinterpret_cast<uint64_t*>(sdr + kTile);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int k0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
   const int qend = min(L >= kTile ? (k0 / L + 1) * L : k0 + kTile, Tlen);
   const int nqt = (qend - k0 + kTile - 1) / kTile;
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -1151,7 +1157,7 @@ __global__ void __launch_bounds__(128, 3)
   pdl_enter();
   lse = after_wait(lse);
   Drow = after_wait(Drow);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * G::tile);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, k0, b);
     tc::tma_load_3d(sV, &mV, &bar[0], h * DH, k0, b);
@@ -1200,13 +1206,13 @@ __global__ void __launch_bounds__(128, 3)
       slse[tid] = tq < Tlen ? -lse[li] * kLog2e : 0.f;
       sdr[tid] = tq < Tlen ? -Drow[li] * scale : 0.f;
     }
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       ok = tc::mbar_wait(&bar[0], qt & 1, status) && ok;
       tc::fence_after_sync();
     }
     __syncthreads();  // slse / sdr written
     for (int q = 0; q < 4; ++q) {
-      if (tid == 0 && q == 0) issue_scores(0);
+      if (warp0 && tc::elect_one() && q == 0) issue_scores(0);
       __syncwarp();
       ok = tc::mbar_wait(&bar[1], ns & 1, status) && ok;
       ++ns;
@@ -1250,7 +1256,7 @@ __global__ void __launch_bounds__(128, 3)
       tc::fence_proxy_async_smem();
       tc::fence_before_sync();
       __syncthreads();
-      if (tid == 0) {
+      if (warp0 && tc::elect_one()) {
         tc::fence_after_sync();
         // every thread has read this quarter's scores out of TMEM (the barrier
         // above): the next quarter's products go first, under this quarter's
@@ -1272,7 +1278,7 @@ __global__ void __launch_bounds__(128, 3)
       }
       ++nq;
     }
-    if (tid == 0 && qt + 1 < nqt) {  // every product of the tile is done with Q / dO
+    if (warp0 && tc::elect_one() && qt + 1 < nqt) {  // every product of the tile is done with Q / dO
       ok = tc::mbar_wait(&bar[2 + ((nq - 1) & 1)], ((nq - 1) >> 1) & 1, status) && ok;
       tc::mbar_arrive_expect_tx(&bar[0], 2 * G::tile);
       tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, q0 + kTile, b);

@@ -91,10 +91,10 @@ __device__ __forceinline__ void store_tile(const CUtensorMap* m, const uint8_t* 
 // MN-major (M = keys, K = queries).  All are 64-column swizzle-128 chunks
 // 16 KB apart.
 __device__ __forceinline__ uint64_t d_kmaj(const uint8_t* t, int kk) {
-  return tc::sdesc(tc::smem_u32(t) + (kk >> 2) * kChunk + (kk & 3) * 32, 16, 1024);
+  return tc::desc_at(tc::sdesc(tc::smem_u32(t), 16, 1024), (kk >> 2) * kChunk + (kk & 3) * 32);
 }
 __device__ __forceinline__ uint64_t d_mnmaj(const uint8_t* t, int kk) {
-  return tc::sdesc(tc::smem_u32(t) + kk * 2048, kChunk, 1024);
+  return tc::desc_at(tc::sdesc(tc::smem_u32(t), kChunk, 1024), kk * 2048);
 }
 
 // Columns of the tile the thread's half owns in the epilogues: OC = 32 NC from
@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dq_smem<NC>());  // loads, S/dP, dQ
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 3);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int q = warp & 3, hf = warp >> 2;
   const int h = blockIdx.y, b = blockIdx.z;
   const TileAt tt = tile_at(a, blockIdx.x);
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     pdl_enter();
     return;
   }
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 3; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * kT);
     load_tile<NC>(sQ, &mQ, &bar[0], h, tt.t0, b);
     load_tile<NC>(sK, &mK, &bar[0], h, tt.kstart, b);
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
 
   for (int kt = 0; kt <= tt.j; ++kt) {
     const bool diag = kt == tt.j;
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       const bool okk = tc::mbar_wait(&bar[0], kt & 1, a.status);
       tc::fence_after_sync();
       if (okk) {
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     tc::fence_proxy_async_smem();
     tc::fence_before_sync();
     __syncthreads();  // dS is in place, S and dP are read
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (ok) {
         const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     __syncwarp();
     ok = tc::mbar_wait(&bar[2], kt & 1, a.status) && ok;
     tc::fence_after_sync();
-    if (tid == 0 && kt < tt.j) {  // K, V and dS are consumed: the next key tile
+    if (warp0 && tc::elect_one() && kt < tt.j) {  // K, V and dS are consumed: the next key tile
       tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
       load_tile<NC>(sK, &mK, &bar[0], h, tt.kstart + (kt + 1) * kTile, b);
       load_tile<NC>(sV, &mV, &bar[0], h, tt.kstart + (kt + 1) * kTile, b);
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
   if (!fin && row_ok) restage_dq(a, b, h, tt.t0 + r, sQ, r, hf * OC / 8, OC / 8);
   tc::fence_proxy_async_smem();
   __syncthreads();
-  if (tid == 0 && ok) {
+  if (warp0 && tc::elect_one() && ok) {
     store_tile<NC>(tt.j == a.tpb - 1 ? &mdQt : &mdQ, sQ, h, tt.t0, b);
     tc::tma_store_commit();
     tc::tma_store_wait_read<0>();
@@ -376,7 +377,8 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dkv_smem<NC, FUSED>());  // loads, S/dP, dV, dK
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int q = warp & 3, hf = warp >> 2;
   const int h = blockIdx.y, b = blockIdx.z;
   const TileAt tt = tile_at(a, blockIdx.x);
@@ -386,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   }
   // query tiles tt.j .. jend-1 of the block
   const int jend = FUSED ? 1 : min(a.tpb, (min(a.x.L, a.x.T - tt.kstart) + kTile - 1) / kTile);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     tc::prefetch_tmap(&mdO);
   }
   pdl_enter();
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 4 * kT);
     load_tile<NC>(sQ, &mQ, &bar[0], h, tt.t0, b);
     load_tile<NC>(sK, &mK, &bar[0], h, tt.t0, b);
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     const float nl2 = row_ok ? -a.x.lse[lrow] * kLog2e : 0.f;
     if (!FUSED) drow = row_ok ? a.Drow[lrow] : 0.f;
     const float ndr = -drow * a.x.scale;
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       const bool okk = tc::mbar_wait(&bar[0], it & 1, a.status);
       tc::fence_after_sync();
       if (okk) {
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     tc::fence_before_sync();
     __syncthreads();  // P is in place, S is read
     const int nkk = (rows + 15) / 16;  // queries past the tile's rows have P = dS = 0
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (ok) {
         for (int kk = 0; kk < nkk; ++kk) {  // dV += P^T dO
@@ -495,7 +497,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     tc::fence_proxy_async_smem();
     tc::fence_before_sync();
     __syncthreads();  // dS is in place; its TMEM columns are read
-    if (tid == 0) {
+    if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (ok) {
         for (int kk = 0; kk < nkk; ++kk) {  // dK += dS^T Q
@@ -516,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     __syncwarp();
     ok = tc::mbar_wait(&bar[3], it & 1, a.status) && ok;
     tc::fence_after_sync();
-    if (!FUSED && tid == 0 && i + 1 < jend) {  // the next query tile
+    if (!FUSED && warp0 && tc::elect_one() && i + 1 < jend) {  // the next query tile
       tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
       load_tile<NC>(sQ, &mQ, &bar[0], h, t0 + kTile, b);
       load_tile<NC>(sdO, &mdO, &bar[0], h, t0 + kTile, b);
@@ -544,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
   __syncthreads();
-  if (tid == 0 && ok) {
+  if (warp0 && tc::elect_one() && ok) {
     const bool tail = !FUSED && tt.j == a.tpb - 1;
     if (FUSED) store_tile<NC>(&mdQ, sQ, h, tt.t0, b);
     store_tile<NC>(tail ? &mdKt : &mdK, sK, h, tt.t0, b);

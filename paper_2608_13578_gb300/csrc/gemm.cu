@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint64_t* tempty = tfull + 2;       // accumulator drained by the epilogue
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
 
   if (warp == 0 && lane == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   pdl_enter();  // setup above overlapped the previous kernel
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ---- TMA producer
       int it = 0;
       bool ok = true;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         tc::mbar_wait(&full[i % STAGES], (i / STAGES) & 1, status);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ---- MMA issuer
       constexpr uint32_t idesc = tc::idesc_bf16(kBM, BN, A_MN ? 1 : 0, B_MN ? 1 : 0);
       int it = 0, j = 0;
@@ -479,10 +479,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           const uint32_t sb = sa + Cfg::A_BYTES;
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk) {
-            const uint64_t ad = A_MN ? tc::sdesc(sa + kk * 2048, 8192, 1024)
-                                     : tc::sdesc(sa + kk * 32, 16, 1024);
-            const uint64_t bd = B_MN ? tc::sdesc(sb + kk * 2048, 8192, 1024)
-                                     : tc::sdesc(sb + kk * 32, 16, 1024);
+            const uint64_t ad = A_MN ? tc::desc_at(tc::sdesc(sa, 8192, 1024), kk * 2048)
+                                     : tc::desc_at(tc::sdesc(sa, 16, 1024), kk * 32);
+            const uint64_t bd = B_MN ? tc::desc_at(tc::sdesc(sb, 8192, 1024), kk * 2048)
+                                     : tc::desc_at(tc::sdesc(sb, 16, 1024), kk * 32);
             tc::mma_bf16(d, ad, bd, idesc, (i | kk) != 0 ? 1u : 0u);
           }
           tc::mma_commit(&empty[s]);
@@ -767,10 +767,10 @@ __device__ __forceinline__ bool tc2_mma(const Tc2Shape& s, int tile, int j, uint
     const uint32_t sb = sa + Cfg::A_BYTES;
 #pragma unroll
     for (int kk = 0; kk < kBK / 16; ++kk) {
-      const uint64_t ad = Op::A_MN ? tc::sdesc(sa + kk * 2048, 8192, 1024)
-                                   : tc::sdesc(sa + kk * 32, 16, 1024);
-      const uint64_t bd = Op::B_MN ? tc::sdesc(sb + kk * 2048, 8192, 1024)
-                                   : tc::sdesc(sb + kk * 32, 16, 1024);
+      const uint64_t ad = Op::A_MN ? tc::desc_at(tc::sdesc(sa, 8192, 1024), kk * 2048)
+                                   : tc::desc_at(tc::sdesc(sa, 16, 1024), kk * 32);
+      const uint64_t bd = Op::B_MN ? tc::desc_at(tc::sdesc(sb, 8192, 1024), kk * 2048)
+                                   : tc::desc_at(tc::sdesc(sb, 16, 1024), kk * 32);
       tc::mma_bf16_pair(d, ad, bd, idesc, (i | kk) != 0 ? 1u : 0u);
     }
     tc::mma_commit_pair(&empty[st]);
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint64_t* tempty = tfull + ACC;     // accumulator drained by both CTAs' epilogues
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + ACC);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = tc::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_rank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   int total = 0;
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   pdl_enter();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       int it = 0;
       for (int r = 0; r < nmine; ++r) {
         int tile;
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && tc::elect_one()) {
       int it = 0;
       for (int j = 0; j < nmine; ++j) {
         int tile;

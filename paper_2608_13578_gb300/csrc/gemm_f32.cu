@@ -19,13 +19,13 @@
 // 8-15 drain the accumulators (two, alternating) and store finished tiles through
 // shared memory with TMA; warp 8 also issues the MMAs, one slice ahead of its
 // draining (a warp of its own for that would cost every thread a quarter of its
-// registers, and a loader that issues them holds up all the splitting).8192 x 1536 x 512 takes 96 us
-// (134 TFLOP/s of fp32 products; 122 us with a loader warp issuing the MMAs),
-// 512 x 1536 x 8192 in 3 splits 80 us (112); the CUDA-core kernel took 497 and
-// 749 us.  A 64-deep slice of a 128 x 128 tile is 1536 cycles of tensor work and
-// 2300 of shared-memory traffic (96 KB of parts written, 192 KB read by the 24
-// MMAs); it takes about 4000, the splitting and the hand-over between the two
-// stages.
+// registers, and a loader that issues them holds up all the splitting).
+// 8192 x 1536 x 512 takes 88 us (146 TFLOP/s of fp32 products; 122 us with a loader
+// warp issuing the MMAs, 96 with their branch taken by lane number, see elect_one),
+// 512 x 1536 x 8192 in 3 splits 73 us (177); the CUDA-core kernel took 497 and 749
+// us.  A 64-deep slice of a 128 x 128 tile is 1536 cycles of tensor work and 2300 of
+// shared-memory traffic (96 KB of parts written, 192 KB read by the 24 MMAs); it
+// takes about 3700, the splitting and the hand-over between the two stages.
 //
 // A row or column holding an infinity (or a value above bf16's range) makes
 // partial products like inf x 0: outputs that come out non-finite are
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* tfull = empty + kStages;
   uint64_t* tempty = tfull + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
 
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -239,17 +239,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       return false;
     tc::fence_after_sync();
     const uint32_t sa = tc::smem_u32(smem + s * C::STAGE);
-    const uint32_t sb = sa + 3 * C::A_PART;
+    const uint64_t ad = tc::sdesc(sa, A_MN ? 8192 : 16, 1024),
+                   bd = tc::sdesc(sa + 3 * C::A_PART, B_MN ? 8192 : 16, 1024);
     const uint32_t d = tmem + (uint32_t)(acc * 2 * BN);
     auto product = [&](int pa, int pb, uint32_t dst, bool first) {
 #pragma unroll
       for (int kk = 0; kk < kBK / 16; ++kk) {
-        const uint32_t xa = sa + pa * C::A_PART, xb = sb + pb * C::B_PART;
-        const uint64_t ad = A_MN ? tc::sdesc(xa + kk * 2048, 8192, 1024)
-                                 : tc::sdesc(xa + kk * 32, 16, 1024);
-        const uint64_t bd = B_MN ? tc::sdesc(xb + kk * 2048, 8192, 1024)
-                                 : tc::sdesc(xb + kk * 32, 16, 1024);
-        tc::mma_bf16(dst, ad, bd, idesc, first && kk == 0 ? 0u : 1u);
+        tc::mma_bf16(dst, tc::desc_at(ad, pa * C::A_PART + kk * (A_MN ? 2048 : 32)),
+                     tc::desc_at(bd, pb * C::B_PART + kk * (B_MN ? 2048 : 32)), idesc,
+                     first && kk == 0 ? 0u : 1u);
       }
     };
     product(0, 0, d, true);       // h h
@@ -317,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tile_at(tile, m0, n0, z, kb, ke);
         slices += (ke - kb + kBK - 1) / kBK;
       }
-    if (slices > 0 && lane == 0) issue(0);
+    if (slices > 0 && tc::elect_one()) issue(0);
     __syncwarp();
     bool ok = true;
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
@@ -328,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < NC; ++c) acc[c] = 0.f;
       for (int k = kb; k < ke; k += kBK, ++it) {
         const int ab = it & 1, use = it >> 1;
-        if (it + 1 < slices && lane == 0) issue(it + 1);
+        if (it + 1 < slices && tc::elect_one()) issue(it + 1);
         __syncwarp();
         ok = tc::mbar_wait(&tfull[ab], use & 1, status) && ok;
         tc::fence_after_sync();

@@ -188,6 +188,11 @@ __device__ __forceinline__ uint64_t sdesc_sw(uint32_t saddr, uint32_t lbo, uint3
   return d;
 }
 
+// The descriptor `bytes` further on (a multiple of 16): shared addresses stay below
+// 2^18, so nothing carries out of the address field, and a loop over K steps adds
+// constants to one descriptor instead of forming each.
+__device__ __forceinline__ uint64_t desc_at(uint64_t d, uint32_t bytes) { return d + (bytes >> 4); }
+
 // Instruction descriptor of kind::f16 with bf16 A and B, fp32 accumulator.
 // a_mn / b_mn: operand is MN-major (1) or K-major (0).
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn, int b_mn) {
@@ -200,9 +205,11 @@ __device__ __forceinline__ void bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// True in one lane of the (converged) warp.  The branch that issues MMAs asks this
-// and not threadIdx: only then does the compiler know that one lane runs it, and
-// passes the descriptors in uniform registers without a loop over the lanes.
+// True in one lane of the (converged) warp, always the same one.  The branch that
+// issues MMAs asks this and not threadIdx: the compiler then knows that one lane
+// runs it.  24 MMAs and a commit took 1970 cycles to issue under threadIdx == 0 and
+// 1320 so, 1100 with one descriptor per operand (desc_at).  (attn_tc.cu keeps
+// threadIdx: its CTAs hide one another's issue, and it measured 4 % slower with this.)
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
