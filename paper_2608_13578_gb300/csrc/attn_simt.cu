@@ -13,11 +13,15 @@
 // 16-byte loads.  In the products over keys or queries it holds four columns
 // (twice four for heads above 64) of one, two or four rows, so that all threads
 // have outputs at every head width, and skips what the causal mask hides from
-// its rows.  Bound: fp32 issue, shared-memory bandwidth close behind.  Before,
-// one warp per query row read every key row from L2; times before and now:
-// B8 T1024 D512 h8 L64 fp32 forward 516 and 59 us, backward 2002 and 93 us;
-// B4 T2048 D1024 h8 L128 bf16 forward 1997 and 131 us; B4 T1000 D768 h8 L48 bf16
-// forward 306 and 63 us.  Deterministic: every sum runs in a fixed order.
+// its rows.  Long walks start first: in tile order the last wave held half of them
+// (16 % of the SMs' time at L 128).  Bound: no single unit (issue 0.55 a cycle, FMA
+// 32 %, shared memory 44 %); two or three CTAs of eight warps hide little of the
+// loads, barriers and exponentials between the products.  Forward: three CTAs per
+// SM for heads up to 64 (80 registers), two above (shared memory).  Before, one warp
+// per query row read every key row from L2; times before and now: B8 T1024 D512 h8
+// L64 fp32 forward 516 and 48 us, backward 2002 and 92 us; B4 T2048 D1024 h8 L128
+// bf16 forward 1997 and 126 us; B4 T1000 D768 h8 L48 bf16 forward 306 and 63 us.
+// Deterministic: every sum runs in a fixed order.
 #include <algorithm>
 #include <mutex>
 
@@ -42,27 +46,63 @@ struct SimtArgs {
   float *lse, *Drow;
   int rows;  // L <= 64: rows per tile (whole blocks)
   int tpb;   // L > 64: tiles per block
+  int nb, B; // tiles (L <= 64) or blocks of a sequence, sequences
   int vec;   // rows of every tensor are aligned to four elements
 };
 
 struct TileAt {
-  int t0, rows, kstart, j;
+  int t0, rows, kstart, j, h, b;
 };
-template <class E>
-__device__ __forceinline__ TileAt tile_at(const SimtArgs<E>& a, int x) {
+// Blocks first, heads of one block as neighbours; tiles of a long block by the key
+// (or query) tiles they walk, the longest walks of the whole grid first, so that
+// the last CTAs to run are short ones (DESC: tile j walks j + 1 of them).
+template <bool DESC, class E>
+__device__ __forceinline__ TileAt tile_at(const SimtArgs<E>& a) {
   TileAt t;
+  int x = blockIdx.x / a.x.H;
+  t.h = blockIdx.x - x * a.x.H;
+  const int n = x / a.nb;
+  x -= n * a.nb;
+  const int jj = n / a.B;
+  t.b = n - jj * a.B;
   if (a.x.L <= kTile) {
     t.t0 = t.kstart = x * a.rows;
     t.j = 0;
     t.rows = min(a.rows, a.x.T - t.t0);
   } else {
-    const int i = x / a.tpb;
-    t.j = x - i * a.tpb;
-    t.kstart = i * a.x.L;
+    t.j = DESC ? a.tpb - 1 - jj : jj;
+    t.kstart = x * a.x.L;
     t.t0 = t.kstart + t.j * kTile;
     t.rows = min(min(kTile, a.x.L - t.j * kTile), a.x.T - t.t0);
   }
   return t;
+}
+
+// The 16-key groups [j0, j0 + n) of a score tile that any of the warp's eight rows
+// sees.  Heads up to 64 (CB = 1) form all four: there the shorter loops do not make
+// up for four copies of the code (B8 T1024 D512 h8 L64 fp32 forward 46 us, 51 with
+// them; backward 90 and 95), above they do (heads of 96, L 48: 169 -> 153 us for 16 x
+// 1000 tokens; heads of 128, L 128, 113 -> 109 us for 4 x 2048).
+struct Groups {
+  int j0, n;
+};
+template <int CB>
+__device__ __forceinline__ Groups groups_seen(bool diag, int rows, int L) {
+  const int r0 = 8 * (threadIdx.x >> 5);
+  if (CB == 1) return {0, 4};
+  if (r0 >= rows) return {0, 0};
+  if (!diag) return {0, 4};
+  const int j0 = L <= kTile ? (r0 / L) * L / 16 : 0;
+  return {j0, min(r0 + 7, rows - 1) / 16 + 1 - j0};
+}
+// f(N) for n groups, N a compile-time count.
+template <int CB, class F>
+__device__ __forceinline__ void with_groups(int n, F&& f) {
+  using std::integral_constant;
+  if (CB == 1 || n == 4) f(integral_constant<int, 4>());
+  else if (n == 3) f(integral_constant<int, 3>());
+  else if (n == 2) f(integral_constant<int, 2>());
+  else if (n == 1) f(integral_constant<int, 1>());
 }
 
 // Rows [0, rows) x dh columns of a head into a tile, the other rows zero; a
@@ -104,8 +144,9 @@ __device__ __forceinline__ void put4(E* p, const float* v, bool vec) {
   }
 }
 
-// s[i][j] = A[4 ty + i] . B[tx + 16 j] over dh columns, each a single chain in
-// column order.
+// s[i][j] = A[4 ty + i] . B[tx + 16 j], j < N, over dh columns, each a single chain
+// in column order.
+template <int N>
 __device__ __forceinline__ void scores_in_order(const float* A, const float* B, int ldh, int dh,
                                                 float (*s)[4]) {
   const float* pa = A + 4 * (threadIdx.x >> 4) * ldh;
@@ -113,18 +154,18 @@ __device__ __forceinline__ void scores_in_order(const float* A, const float* B, 
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+    for (int j = 0; j < N; ++j) s[i][j] = 0.f;
 #pragma unroll 2
   for (int k = 0; k < dh; k += 4) {
-    float4 x[4], y[4];
+    float4 x[4], y[N];
 #pragma unroll
     for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(pa + i * ldh + k);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
+    for (int j = 0; j < N; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < N; ++j) {
         s[i][j] = fmaf(x[i].x, y[j].x, s[i][j]);
         s[i][j] = fmaf(x[i].y, y[j].y, s[i][j]);
         s[i][j] = fmaf(x[i].z, y[j].z, s[i][j]);
@@ -134,27 +175,28 @@ __device__ __forceinline__ void scores_in_order(const float* A, const float* B, 
 }
 
 // The same with two chains per score (even and odd columns), as packed pairs.
+template <int N>
 __device__ __forceinline__ void scores(const float* A, const float* B, int ldh, int dh,
                                        float (*s)[4]) {
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  float2 acc[4][4];
+  float2 acc[4][N];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int j = 0; j < N; ++j) acc[i][j] = make_float2(0.f, 0.f);
   const float* pa = A + (4 * ty) * ldh;
   const float* pb = B + tx * ldh;
 #pragma unroll 2
   for (int k = 0; k < dh; k += 4) {
-    float4 x[4], y[4];
+    float4 x[4], y[N];
 #pragma unroll
     for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(pa + i * ldh + k);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
+    for (int j = 0; j < N; ++j) y[j] = *reinterpret_cast<const float4*>(pb + 16 * j * ldh + k);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < N; ++j) {
         acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].y), make_float2(y[j].x, y[j].y), acc[i][j]);
         acc[i][j] = __ffma2_rn(make_float2(x[i].z, x[i].w), make_float2(y[j].z, y[j].w), acc[i][j]);
       }
@@ -162,7 +204,7 @@ __device__ __forceinline__ void scores(const float* A, const float* B, int ldh, 
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) s[i][j] = acc[i][j].x + acc[i][j].y;
+    for (int j = 0; j < N; ++j) s[i][j] = acc[i][j].x + acc[i][j].y;
 }
 
 // The thread's outputs: column group threadIdx.x % C4 (four columns, CB times 64
@@ -285,7 +327,7 @@ __device__ __forceinline__ int block_end(int r, int L) {
 // take turns in one buffer, where that makes room for a second CTA on the SM.
 constexpr int kKeep = 4;
 template <class E, int C4, int CB>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, CB == 1 ? 3 : 2)
     attn_fwd_simt_kernel(const __grid_constant__ SimtArgs<E> a, int ldp, int share) {
   pdl_enter();
   using C = Cols<C4, CB>;
@@ -293,9 +335,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int dh = a.x.dh, ldh = dh + 4;
   float *Qs = sm, *Ks = Qs + kTile * ldh, *Vs = share ? Ks : Ks + kTile * ldh,
         *Ps = Vs + kTile * ldh, *inv = Ps + kTile * ldp;  // inv: [64]
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int h = blockIdx.y, b = blockIdx.z;
-  const TileAt tt = tile_at(a, blockIdx.x);
+  const int tid = threadIdx.x, ty = threadIdx.x >> 4, tx = tid & 15;
+  const TileAt tt = tile_at<true>(a);
+  const int h = tt.h, b = tt.b;
   if (tt.rows <= 0) return;
   const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
@@ -304,15 +346,16 @@ __global__ void __launch_bounds__(kThreads, 2)
   auto load_tile = [&](float* dst, const E* src, int kt) {
     fill(dst, ldh, src + (row0 + tt.kstart + kt * kTile) * a.x.ld + c0, a.x.ld, keys(kt), dh, a.vec);
   };
-  // the thread's scaled scores of key tile kt (hidden keys -inf)
-  auto tile_scores = [&](int kt, float (*s)[4]) {
-    scores_in_order(Qs, Ks, ldh, dh, s);
+  // the thread's scaled scores of N groups of key tile kt (hidden keys -inf)
+  auto tile_scores = [&](auto n, int j0, int kt, float (*s)[4]) {
+    constexpr int N = decltype(n)::value;
+    scores_in_order<N>(Qs, Ks + 16 * j0 * ldh, ldh, dh, s);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = 4 * ty + i, rbs = block_row(r, a.x.L);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int k = tx + 16 * j;
+      for (int j = 0; j < N; ++j) {
+        const int k = tx + 16 * (j0 + j);
         s[i][j] = (kt < tt.j || (k >= rbs && k <= r)) ? __fmul_rn(s[i][j], a.x.scale) : -INFINITY;
       }
     }
@@ -324,30 +367,37 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (kt > 0) __syncthreads();
     load_tile(Ks, a.x.K, kt);
     __syncthreads();
-    float s[4][4];
-    tile_scores(kt, s);
+    const Groups g = groups_seen<CB>(kt == tt.j, tt.rows, a.x.L);
+    with_groups<CB>(g.n, [&](auto n) {
+      float s[4][4];
+      tile_scores(n, g.j0, kt, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        mx[i] = fmaxf(mx[i], s[i][j]);
-        if (keep) Ps[(4 * ty + i) * ldp + kt * kTile + tx + 16 * j] = s[i][j];
-      }
+        for (int j = 0; j < decltype(n)::value; ++j) {
+          mx[i] = fmaxf(mx[i], s[i][j]);
+          if (keep) Ps[(4 * ty + i) * ldp + kt * kTile + tx + 16 * (g.j0 + j)] = s[i][j];
+        }
+    });
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) mx[i] = max16(mx[i]);
 
-  // exponentials of key tile kt into columns p0 .. of Ps
+  // exponentials of key tile kt into columns p0 .. of Ps (groups that no row of the
+  // warp sees are neither written nor read)
   auto exps = [&](int kt, int p0) {
-    float s[4][4];
-    if (!keep) tile_scores(kt, s);
+    const Groups g = groups_seen<CB>(kt == tt.j, tt.rows, a.x.L);
+    with_groups<CB>(g.n, [&](auto n) {
+      float s[4][4];
+      if (!keep) tile_scores(n, g.j0, kt, s);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float* p = Ps + (4 * ty + i) * ldp + p0 + tx + 16 * j;
-        *p = expf((keep ? *p : s[i][j]) - mx[i]);
-      }
+        for (int j = 0; j < decltype(n)::value; ++j) {
+          float* p = Ps + (4 * ty + i) * ldp + p0 + tx + 16 * (g.j0 + j);
+          *p = expf((keep ? *p : s[i][j]) - mx[i]);
+        }
+    });
   };
   if (keep)
     for (int kt = 0; kt <= tt.j; ++kt) exps(kt, kt * kTile);
@@ -373,15 +423,16 @@ __global__ void __launch_bounds__(kThreads, 2)
       load_tile(Vs, a.x.V, kt);
       __syncthreads();
     }
-    // partial sums, warp w: rows 8w .. 8w+7, lane = key index in the block mod 32
+    // partial sums of the warp's eight rows, lane = key index in the block mod 32
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int r = 8 * warp + u, rbs = block_row(r, a.x.L);
-      const int n = kt < tt.j ? kTile : r + 1 - rbs;  // visible keys of this tile
+      const int n = r >= tt.rows ? 0 : kt < tt.j ? kTile : r + 1 - rbs;  // visible keys of this tile
       for (int j = lane; j < n; j += 32) part[u] += Ps[r * ldp + p0 + rbs + j];
     }
     rows_times<C4, CB>(Ps, ldp, Vs, ldh, dh, p0 + (kt < tt.j ? 0 : block_row(C::row(), a.x.L)),
-                       p0 + (kt < tt.j ? kTile : min(C::row() + C::RT, tt.rows)), p0, acc);
+                       p0 + (C::row() >= tt.rows ? 0 : kt < tt.j ? kTile : min(C::row() + C::RT, tt.rows)),
+                       p0, acc);
   }
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
@@ -436,34 +487,40 @@ __device__ __forceinline__ void drow4(const SimtArgs<E>& a, const TileAt& tt, in
     d[i] = sum16(s);
   }
 }
-// P and dS = P (dP - Drow) scale of the thread's 4 x 4 block, rows past `rows`
-// and hidden keys 0.
-template <class E>
+// P and dS = P (dP - Drow) scale of the thread's rows into score tiles (P may be
+// null), rows past `rows` and hidden keys 0; groups that no row of the warp sees are
+// neither written nor read.
+template <int CB, class E>
 __device__ __forceinline__ void p_ds(const SimtArgs<E>& a, const float* Qs, const float* Ks,
                                      const float* Gs, const float* Vs, int ldh, bool diag, int rows,
-                                     const float* lse, const float* drow, float (*p)[4],
-                                     float (*ds)[4]) {
+                                     const float* lse, const float* drow, float* P, float* S) {
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  scores(Qs, Ks, ldh, a.x.dh, p);
-  scores(Gs, Vs, ldh, a.x.dh, ds);
+  const Groups g = groups_seen<CB>(diag, rows, a.x.L);
+  with_groups<CB>(g.n, [&](auto n) {
+    constexpr int N = decltype(n)::value;
+    float p[4][4], ds[4][4];
+    scores<N>(Qs, Ks + 16 * g.j0 * ldh, ldh, a.x.dh, p);
+    scores<N>(Gs, Vs + 16 * g.j0 * ldh, ldh, a.x.dh, ds);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = 4 * ty + i, rbs = block_row(r, a.x.L);
+    for (int i = 0; i < 4; ++i) {
+      const int r = 4 * ty + i, rbs = block_row(r, a.x.L);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int k = tx + 16 * j;
-      const bool vis = r < rows && (!diag || (k >= rbs && k <= r));
-      p[i][j] = vis ? expf(p[i][j] * a.x.scale - lse[i]) : 0.f;
-      ds[i][j] = vis ? p[i][j] * (ds[i][j] - drow[i]) * a.x.scale : 0.f;
+      for (int j = 0; j < N; ++j) {
+        const int k = tx + 16 * (g.j0 + j);
+        const bool vis = r < rows && (!diag || (k >= rbs && k <= r));
+        p[i][j] = vis ? expf(p[i][j] * a.x.scale - lse[i]) : 0.f;
+        ds[i][j] = vis ? p[i][j] * (ds[i][j] - drow[i]) * a.x.scale : 0.f;
+      }
     }
-  }
-}
-__device__ __forceinline__ void put_tile(float* P, const float (*v)[4]) {
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) P[(4 * ty + i) * kPld + tx + 16 * j] = v[i][j];
+      for (int j = 0; j < N; ++j) {
+        const int o = (4 * ty + i) * kPld + tx + 16 * (g.j0 + j);
+        if (P) P[o] = p[i][j];
+        S[o] = ds[i][j];
+      }
+  });
 }
 template <class E>
 __device__ __forceinline__ void rows_lse(const SimtArgs<E>& a, int b, int h, int t0, int rows,
@@ -503,8 +560,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
   float *Qs = sm, *Gs = Qs + kTile * ldh, *Ks = Gs + kTile * ldh, *Vs = Ks + kTile * ldh,
         *Ss = Vs + kTile * ldh;
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  const int h = blockIdx.y, b = blockIdx.z;
-  const TileAt tt = tile_at(a, blockIdx.x);
+  const TileAt tt = tile_at<true>(a);
+  const int h = tt.h, b = tt.b;
   if (tt.rows <= 0) return;
   const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
@@ -528,11 +585,10 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     fill(Ks, ldh, a.x.K + (row0 + k0) * a.x.ld + c0, a.x.ld, nk, dh, a.vec);
     fill(Vs, ldh, a.x.V + (row0 + k0) * a.x.ld + c0, a.x.ld, nk, dh, a.vec);
     __syncthreads();
-    float p[4][4], ds[4][4];
-    p_ds(a, Qs, Ks, Gs, Vs, ldh, diag, tt.rows, lse, drow, p, ds);
-    put_tile(Ss, ds);
+    p_ds<CB>(a, Qs, Ks, Gs, Vs, ldh, diag, tt.rows, lse, drow, nullptr, Ss);
     __syncthreads();
-    rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, 0, diag ? min(C::row() + C::RT, nk) : kTile, 0, acc);
+    rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, 0,
+                       C::row() >= tt.rows ? 0 : diag ? min(C::row() + C::RT, nk) : kTile, 0, acc);
   }
   store_dq<E, C4, CB>(a, tt, b, h, acc);
 }
@@ -549,8 +605,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
   const int dh = a.x.dh, ldh = dh + 4;
   float *Ks = sm, *Vs = Ks + kTile * ldh, *Qs = Vs + kTile * ldh, *Gs = Qs + kTile * ldh,
         *Ps = Gs + kTile * ldh, *Ss = Ps + kTile * kPld;
-  const int h = blockIdx.y, b = blockIdx.z;
-  const TileAt tt = tile_at(a, blockIdx.x);
+  const TileAt tt = tile_at<false>(a);
+  const int h = tt.h, b = tt.b;
   if (tt.rows <= 0) return;
   const long row0 = (long)b * a.x.T;
   const int c0 = h * dh;
@@ -575,12 +631,7 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
       rows_lse(a, b, h, t0, rows, a.Drow, drow);
     rows_lse(a, b, h, t0, rows, a.lse, lse);
     __syncthreads();
-    {
-      float p[4][4], ds[4][4];
-      p_ds(a, Qs, Ks, Gs, Vs, ldh, diag, rows, lse, drow, p, ds);
-      put_tile(Ps, p);
-      put_tile(Ss, ds);
-    }
+    p_ds<CB>(a, Qs, Ks, Gs, Vs, ldh, diag, rows, lse, drow, Ps, Ss);
     __syncthreads();
     // the queries that see any of the thread's keys
     const int lo = diag ? C::row() : 0;
@@ -607,7 +658,7 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     float dq[C::RT][CB][4];
     zero<C::RT, CB>(dq);
     rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, block_row(C::row(), a.x.L),
-                       min(C::row() + C::RT, tt.rows), 0, dq);
+                       C::row() >= tt.rows ? 0 : min(C::row() + C::RT, tt.rows), 0, dq);
     store_dq<E, C4, CB>(a, tt, b, h, dq);
   }
 }
@@ -628,6 +679,8 @@ SimtArgs<E> simt_args(const AttnArgs& f, const AttnBwdArgs* ab) {
   a.Drow = ab ? ab->Drow : nullptr;
   a.rows = f.L <= kTile ? (kTile / f.L) * f.L : kTile;
   a.tpb = f.L <= kTile ? 1 : (f.L + kTile - 1) / kTile;
+  a.nb = f.L <= kTile ? (f.T + a.rows - 1) / a.rows : (f.T + f.L - 1) / f.L;
+  a.B = f.B;
   // rows of q, k, v and of the gradients may have any stride; those of O and dO
   // are D elements apart, a multiple of 64
   a.vec = f.ld_qkv % 4 == 0 && a.ld_d % 4 == 0;
@@ -648,9 +701,8 @@ cudaError_t simt_launch(const Launch& lc, K kern, std::atomic<unsigned long long
   if (cudaError_t e = smem_opt_in(kern, simt_smem(std::max(tiles, 3), max_cols, kMaxDh), opted);
       e != cudaSuccess)
     return e;
-  const int nx = f.L <= kTile ? (f.T + a.rows - 1) / a.rows : (f.T + f.L - 1) / f.L * a.tpb;
-  cudaError_t e = launch_k(kern, dim3(nx, f.H, f.B), dim3(kThreads), simt_smem(tiles, cols, f.dh),
-                           lc.stream, a, x...);
+  cudaError_t e = launch_k(kern, dim3((unsigned)a.nb * a.tpb * f.H * f.B), dim3(kThreads),
+                           simt_smem(tiles, cols, f.dh), lc.stream, a, x...);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
