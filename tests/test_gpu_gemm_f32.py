@@ -16,9 +16,9 @@ from tests.test_gpu_kernels import LAYOUTS, _operand
 pytestmark = pytest.mark.gpu
 
 # tile edges (128 rows, 64 / 128 columns, 64-deep slices), one row, and enough
-# tiles for several per CTA
+# tiles for several per CTA (within and past the eight slices that share an accumulator)
 SHAPES = [(128, 64, 64), (256, 384, 128), (1, 64, 512), (136, 192, 72), (1000, 512, 520),
-          (8, 128, 1536), (6144, 768, 256)]
+          (8, 128, 1536), (6144, 768, 256), (6144, 768, 584)]
 
 
 @pytest.fixture(scope="module")
