@@ -14,7 +14,11 @@
 // through a TMA store.  The backward recomputes P from the saved log-sum-exp
 // and runs the five products S = Q K^T, dP = dO V^T, dV = P^T dO,
 // dQ = dS K, dK = dS^T Q on the tensor cores, reading the same shared tiles
-// K-major or MN-major as each product needs.
+// K-major or MN-major as each product needs.  MMAs are issued under elect_one()
+// (tc.cuh): forward / backward 6.8 -> 6.4 / 13.6 -> 13.3 us at B8 T1024 L64 D512 h8,
+// 9.4 -> 8.7 / 15.2 -> 14.6 us at B16 T1024 L64 D128 h8 (bound: the chain load, MMA,
+// softmax, MMA of each tile), 124.5 -> 123.8 / 225 -> 222 us at B4 T16384 L128 D1024
+// h16 (0.64 and 0.71 of HBM bandwidth).
 #include "attn_common.cuh"
 #include "common.cuh"
 #include "internal.h"
@@ -67,12 +71,13 @@ __global__ void __launch_bounds__(128)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (DH == 64 ? 3 * kT : 3 * kT + 32768));
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
 
   // Setup overlaps the previous kernel (before pdl_wait); the loads go out
   // first after it, so the TMEM allocation and the block barrier overlap them.
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 3; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -80,7 +85,7 @@ __global__ void __launch_bounds__(128)
     tc::prefetch_tmap(&mV);
   }
   pdl_enter();
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 3 * kT);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, t0, b);
@@ -97,7 +102,7 @@ __global__ void __launch_bounds__(128)
   const uint32_t tmem = *tslot;
   const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     const bool ok = tc::mbar_wait(&bar[0], 0, status);
     tc::fence_after_sync();
     if (ok) {
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(128)
   tc::fence_before_sync();
   __syncthreads();
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::fence_after_sync();
     constexpr uint32_t idO = tc::idesc_bf16(128, DH, 0, 1);
 #pragma unroll
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(128)
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
   __syncthreads();
-  if (tid == 0 && ok) {
+  if (warp0 && tc::elect_one() && ok) {
     tc::tma_store_3d(&mO, sQ, h * DH, t0, b);
     tc::tma_store_commit();
     tc::tma_store_wait_read<0>();  // the staging is read; the writes finish with the grid
@@ -231,10 +236,11 @@ __global__ void __launch_bounds__(128)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + (DH == 64 ? 6 * kT : 5 * kT + 32768));
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const bool warp0 = warp == 0;
   const int t0 = blockIdx.x * kTile, h = blockIdx.y, b = blockIdx.z;
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(&bar[i], 1);
     tc::fence_mbar_init();
     tc::prefetch_tmap(&mQ);
@@ -245,7 +251,7 @@ __global__ void __launch_bounds__(128)
   }
   pdl_enter();
   lse = after_wait(lse);
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::mbar_arrive_expect_tx(&bar[0], 5 * kT);
     tc::tma_load_3d(sQ, &mQ, &bar[0], h * DH, t0, b);
     tc::tma_load_3d(sK, &mK, &bar[0], h * DH, t0, b);
@@ -264,7 +270,7 @@ __global__ void __launch_bounds__(128)
   const uint32_t tmem = *tslot;
   const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     const bool ok = tc::mbar_wait(&bar[0], 0, status);
     tc::fence_after_sync();
     if (ok) {
@@ -350,13 +356,13 @@ __global__ void __launch_bounds__(128)
   tc::fence_before_sync();
   __syncthreads();
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::fence_after_sync();
     // dV = P^T dO -> columns 0.. (A = P read MN-major: M = keys, K = queries)
     constexpr uint32_t idMN = tc::idesc_bf16(128, DH, 1, 1);
 #pragma unroll
     for (int kk = 0; kk < kTile / 16; ++kk)
-      tc::mma_bf16(tmem, tc::sdesc(tc::smem_u32(sP) + kk * 2048, 16384, 1024),
+      tc::mma_bf16(tmem, tc::desc_at(tc::sdesc(tc::smem_u32(sP), 16384, 1024), kk * 2048),
                    G::mnmaj(sdO, 0, kk), idMN, kk > 0 ? 1u : 0u);
     tc::mma_commit(&bar[2]);
   }
@@ -379,15 +385,15 @@ __global__ void __launch_bounds__(128)
   tc::fence_before_sync();
   __syncthreads();
 
-  if (tid == 0) {
+  if (warp0 && tc::elect_one()) {
     tc::fence_after_sync();
     const uint32_t adS = tc::smem_u32(sP);
     // dK = dS^T Q -> columns 64..
     constexpr uint32_t idMN = tc::idesc_bf16(128, DH, 1, 1);
 #pragma unroll
     for (int kk = 0; kk < kTile / 16; ++kk)
-      tc::mma_bf16(tmem + 64, tc::sdesc(adS + kk * 2048, 16384, 1024), G::mnmaj(sQ, 0, kk), idMN,
-                   kk > 0 ? 1u : 0u);
+      tc::mma_bf16(tmem + 64, tc::desc_at(tc::sdesc(adS, 16384, 1024), kk * 2048),
+                   G::mnmaj(sQ, 0, kk), idMN, kk > 0 ? 1u : 0u);
     // dQ = dS K -> columns 128.. (A = dS K-major, B = K read MN-major)
     constexpr uint32_t idKM = tc::idesc_bf16(128, DH, 0, 1);
 #pragma unroll
@@ -412,7 +418,7 @@ __global__ void __launch_bounds__(128)
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
   __syncthreads();
-  if (tid == 0 && ok) {
+  if (warp0 && tc::elect_one() && ok) {
     tc::tma_store_3d(&mdQ, sQ, h * DH, t0, b);
     tc::tma_store_3d(&mdK, sK, h * DH, t0, b);
     tc::tma_store_3d(&mdV, sdO, h * DH, t0, b);

@@ -208,8 +208,7 @@ __device__ __forceinline__ void bar_sync(int id, int n) {
 // True in one lane of the (converged) warp, always the same one.  The branch that
 // issues MMAs asks this and not threadIdx: the compiler then knows that one lane
 // runs it.  24 MMAs and a commit took 1970 cycles to issue under threadIdx == 0 and
-// 1320 so, 1100 with one descriptor per operand (desc_at).  (attn_tc.cu keeps
-// threadIdx: its CTAs hide one another's issue, and it measured 4 % slower with this.)
+// 1320 so, 1100 with one descriptor per operand (desc_at).
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
