@@ -233,8 +233,9 @@ KERNEL_SOURCES = {
     "attn_bwd_tc": ("attn_tc.cu", "attn_common.cuh"),
     "attn_fwd_fl": ("attn_flash.cu", "attn_common.cuh"),
     "attn_bwd_fl": ("attn_blk.cu", "attn_flash.cu", "attn_common.cuh"),
-    "attn_fwd_simt": ("attn_simt.cu",),
-    "attn_bwd_simt": ("attn_simt.cu",),
+    "attn_bwd_gen": ("attn_gen.cu", "attn_slow.cuh", "attn_common.cuh"),
+    "attn_fwd_simt": ("attn_simt.cu", "attn_slow.cuh"),
+    "attn_bwd_simt": ("attn_simt.cu", "attn_slow.cuh"),
 }
 
 

@@ -25,8 +25,8 @@
 // -> dK, dQ of one CTA, several microseconds, covered by a second CTA per SM
 // where shared memory allows (heads up to 64).  Against the CUDA-core kernels
 // that served these shapes before (one warp per row, operands re-read from L2
-// per row): B4 T2048 D1024 heads of 128 L128 8230 -> 81 us, B4 T1000 D768 heads
-// of 96 L48 1161 -> 49 us.
+// per row): B4 T2048 D1024 heads of 128 L128 8230 -> 76 us, B4 T1000 D768 heads
+// of 96 L48 1161 -> 45 us.
 //
 // A masked key's weight is exactly 0, but 0 x inf = NaN in the products: a row
 // whose result is not finite is recomputed from its visible keys alone
