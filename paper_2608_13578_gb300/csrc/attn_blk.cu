@@ -17,20 +17,22 @@
 //              are free, then the pair's three gradient products;
 //   warp 9     stores finished tiles and loads the next block's into their place, so
 //              a block's first loads run under the last one's work;
-//   warps 10, 11  the next block's row statistics (Drow = dO . O); the first block's
-//              come from warps 0-7.
+//   warps 10, 11  a tile's row statistics (Drow = dO . O) as soon as its slot is
+//              loaded, from the O and dO tiles in shared memory (O through one buffer
+//              of its own).  Read from global memory, a row a thread, they took as
+//              long as all the rest: B16 T1024 D768 h12 L256 73 us, 65 so.
 //
 // What bounds it: a pair's 26 or more MMAs and their issue (about 1700 cycles at DH =
 // 16) next to the elementwise chain (1400: 64 exponentials a thread, 64 KB of stores),
 // the two overlapping but for the first pair of a block; at DH = 64, also the loads.
-// Per pair 1.5 us at DH = 16, 4.2 us at DH = 64 (L 256, HBM's share 1.9 us).  The
+// Per pair 1.4 us at DH = 16, 3.9 us at DH = 64 (L 256, HBM's share 1.9 us).  The
 // two-kernel form (attn_flash.cu, which keeps the shapes that do not fit) forms S and
 // dP once for dQ and once more for dK, dV, and is the slower one from the smallest
 // grid on: in us, two kernels -> this, for 8 / 152 / 608 (block, head)s:
-//   DH 16, L 256    23 -> 15    27 -> 15    64 -> 34
-//   DH 16, L 1024   64 -> 62   148 -> 64   470 -> 218
-//   DH 32, L 512    42 -> 27    74 -> 31   206 -> 83
-//   DH 64, L 256    25 -> 19    36 -> 25   115 -> 56
+//   DH 16, L 256     21 -> 13      27 -> 15      62 -> 33
+//   DH 16, L 1024    57 -> 56     139 -> 60     441 -> 206
+//   DH 32, L 512     38 -> 25      70 -> 27     195 -> 78
+//   DH 64, L 256     25 -> 15      36 -> 21     111 -> 50
 #include "attn_common.cuh"
 #include "common.cuh"
 #include "internal.h"
@@ -49,8 +51,6 @@ constexpr int kThreads = 384;
 constexpr int kMaxM = 8;
 
 struct BlkArgs {
-  const bf16 *O, *dO;
-  long ld_o;
   const float* lse;
   float* Drow;
   int T, H, L, m;
@@ -59,10 +59,10 @@ struct BlkArgs {
   unsigned* status;
 };
 
-// P and dS (32 KB each), m tiles of Q and of dO, two of K and of V, two blocks' row
+// P and dS (32 KB each), m tiles of Q and of dO, two of K and of V, one of O, the row
 // statistics, barriers.
 template <int DH> constexpr int blk_smem(int m) {
-  return 1024 + 65536 + (2 * m + 4) * (int)Geo<DH>::tile + 2 * m * kTile * 8 + 256;
+  return 1024 + 65536 + (2 * m + 5) * (int)Geo<DH>::tile + m * kTile * 8 + 384;
 }
 
 // Item it: heads of one block are neighbours (their rows share memory pages).
@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     attn_bwd_blk_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
                         const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO,
                         const __grid_constant__ CUtensorMap mdQ, const __grid_constant__ CUtensorMap mdK,
-                        const __grid_constant__ CUtensorMap mdV, const __grid_constant__ BlkArgs a) {
+                        const __grid_constant__ CUtensorMap mdV, const __grid_constant__ CUtensorMap mO,
+                        const __grid_constant__ BlkArgs a) {
   using G = Geo<DH>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -101,15 +102,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* sdO = sQ + a.m * G::tile;     // m tiles; dV likewise
   uint8_t* sK = sdO + a.m * G::tile;     // two; dK likewise
   uint8_t* sV = sK + 2 * G::tile;        // two
-  float2* stat = reinterpret_cast<float2*>(sV + 2 * G::tile);  // [2][m * 128]: -lse log2 e, -Drow scale
-  // Barriers in pairs are used in turn; c counts a CTA's key tiles, p its pairs and
-  // n its items, over all items.
-  uint64_t* bar_q = reinterpret_cast<uint64_t*>(stat + 2 * a.m * kTile);  // [8] Q, dO tile loaded
+  uint8_t* sO = sV + 2 * G::tile;        // one
+  float2* stat = reinterpret_cast<float2*>(sO + G::tile);  // [m * 128]: -lse log2 e, -Drow scale
+  // Barriers in pairs are used in turn; c counts a CTA's key tiles, p its pairs and o
+  // its query tiles, over all items.  Slots and statistics need no "free" barrier of
+  // their own: a slot is loaded again, and its rows' statistics formed, only after
+  // the gradients of its tile are stored.
+  uint64_t* bar_q = reinterpret_cast<uint64_t*>(stat + a.m * kTile);  // [8] Q, dO tile loaded
   uint64_t* bar_k = bar_q + kMaxM;  // [2] K, V of key tile c loaded
   uint64_t* bar_e = bar_k + 2;      // [2] gradients of key tile c staged (8 warps)
-  uint64_t* bar_t = bar_e + 2;      // [2] row statistics of item n written (2 warps)
-  uint64_t* bar_d = bar_t + 2;      // [2] row statistics of item n read (8 warps)
-  uint64_t* bar_s = bar_d + 2;      // S, dP of pair p
+  uint64_t* bar_t = bar_e + 2;      // [8] row statistics of a tile written (2 warps)
+  uint64_t* bar_o = bar_t + kMaxM;  // O of query tile o loaded
+  uint64_t* bar_s = bar_o + 1;      // S, dP of pair p
   uint64_t* bar_g = bar_s + 1;      // gradient products of pair p
   uint64_t* bar_r = bar_g + 1;      // S and dP of pair p in registers (8 warps)
   uint64_t* bar_p = bar_r + 1;      // P and dS of pair p in shared memory (8 warps)
@@ -120,13 +124,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int step = gridDim.x;
 
   if (warp == 0 && tc::elect_one()) {
-    for (int i = 0; i < kMaxM; ++i) tc::mbar_init(&bar_q[i], 1);
+    for (int i = 0; i < kMaxM; ++i) {
+      tc::mbar_init(&bar_q[i], 1);
+      tc::mbar_init(&bar_t[i], kStatThreads / 32);
+    }
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&bar_k[i], 1);
       tc::mbar_init(&bar_e[i], kWorkers / 32);
-      tc::mbar_init(&bar_t[i], kStatThreads / 32);
-      tc::mbar_init(&bar_d[i], kWorkers / 32);
     }
+    tc::mbar_init(bar_o, 1);
     tc::mbar_init(bar_s, 1);
     tc::mbar_init(bar_g, 1);
     tc::mbar_init(bar_r, kWorkers / 32);
@@ -143,30 +149,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = *tslot;
   pdl_enter();
   bool ok = true;
-  // Statistics of an item's rows by n threads: Drow = dO . O, and what P and dS take.
-  auto row_stats = [&](const Item& j, float2* dst, int i, int n) {
-    const bf16 *O = after_wait(a.O), *dO = after_wait(a.dO);
-    const float* lse = after_wait(a.lse);
-    for (; i < j.nq * kTile; i += n) {
-      float2 st = make_float2(0.f, 0.f);
-      if (j.t0 + i < a.T) {
-        const long row = (long)j.b * a.T + j.t0 + i, o = row * a.ld_o + j.h * DH;
-        const long li = ((long)j.b * a.H + j.h) * a.T + j.t0 + i;
-        float d = 0.f;
-#pragma unroll
-        for (int u = 0; u < DH / 8; ++u) {
-          float ov[8], gv[8];
-          load8(O + o + 8 * u, ov);
-          load8(dO + o + 8 * u, gv);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) d = fmaf(ov[e], gv[e], d);
-        }
-        a.Drow[li] = d;
-        st = make_float2(-lse[li] * kLog2e, -d * a.scale);
-      }
-      dst[i] = st;
-    }
-  };
 
   if (warp == kMmaWarp) {
     // ------------------------------------------------------------ products
@@ -289,13 +271,67 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp >= kStatWarp) {
-    // ------------------------------------------------ the next items' statistics
-    int n = 0;
-    for (int it = blockIdx.x; it < a.total; it += step, ++n) {
-      if (n >= 2) ok = ok && tc::mbar_wait(&bar_d[n & 1], ((n >> 1) - 1) & 1, a.status);
-      if (n > 0) row_stats(Item(a, it), stat + (n & 1) * a.m * kTile, tid - kStatWarp * 32, kStatThreads);
+    // ------------------------------------- row statistics, from the O and dO tiles
+    const float* lse = after_wait(a.lse);
+    const int w = tid - kStatWarp * 32;
+    struct At {  // a query tile of the CTA's items
+      int it, qt;
+    };
+    auto after = [&](At t) {
+      if (++t.qt == Item(a, t.it).nq) t = {t.it + step, 0};
+      return t;
+    };
+    // its O on the way to shared memory and its log-sum-exp into v
+    auto fetch = [&](At t, float* v) {
+      if (t.it >= a.total) return;
+      const Item j(a, t.it);
+      const int r0 = j.t0 + t.qt * kTile;
+      if (warp == kStatWarp && tc::elect_one() && ok) {
+        tc::mbar_arrive_expect_tx(bar_o, G::tile);
+        tc::tma_load_3d(sO, &mO, bar_o, j.h * DH, r0, j.b);
+      }
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&bar_t[n & 1]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = r0 + w + u * kStatThreads;
+        v[u] = i < a.T ? lse[((long)j.b * a.H + j.h) * a.T + i] : 0.f;
+      }
+    };
+    uint32_t qph = 0;
+    At t{(int)blockIdx.x, 0};
+    float ls[2] = {0.f, 0.f};
+    fetch(t, ls);
+    for (int o = 0; t.it < a.total; ++o) {
+      const Item j(a, t.it);
+      ok = ok && tc::mbar_wait(bar_o, o & 1, a.status);
+      ok = ok && tc::mbar_wait(&bar_q[t.qt], (qph >> t.qt) & 1, a.status);
+      qph ^= 1u << t.qt;
+      const uint8_t* g = sdO + t.qt * G::tile;
+      float d[2] = {0.f, 0.f};
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int k = 0; k < DH / 8; ++k) {
+          float ov[8], gv[8];
+          load8(reinterpret_cast<const bf16*>(sO + G::unit(w + u * kStatThreads, k)), ov);
+          load8(reinterpret_cast<const bf16*>(g + G::unit(w + u * kStatThreads, k)), gv);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) d[u] = fmaf(ov[e], gv[e], d[u]);
+        }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = t.qt * kTile + w + u * kStatThreads;
+        float2 st = make_float2(0.f, 0.f);
+        if (j.t0 + i < a.T) {
+          a.Drow[((long)j.b * a.H + j.h) * a.T + j.t0 + i] = d[u];
+          st = make_float2(-ls[u] * kLog2e, -d[u] * a.scale);
+        }
+        stat[i] = st;
+      }
+      tc::bar_sync(2, kStatThreads);  // O is read
+      if (lane == 0) tc::mbar_arrive(&bar_t[t.qt]);
+      t = after(t);
+      fetch(t, ls);
     }
   } else {
     // ------------------------------------------------- elementwise, results
@@ -304,19 +340,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = q * 32 + lane;
     const float sl2 = a.scale * kLog2e;
     const float2 sl2x2 = make_float2(sl2, sl2), sc2 = make_float2(a.scale, a.scale);
-    int p = 0, c = 0, n = 0;
-    for (int it = blockIdx.x; it < a.total; it += step, ++n) {
+    uint32_t tph = 0;  // parity of each tile's next statistics
+    int p = 0, c = 0;
+    for (int it = blockIdx.x; it < a.total; it += step) {
       const int nq = Item(a, it).nq;
-      const float2* rs = stat + (n & 1) * a.m * kTile + r;
-      if (n == 0) {  // nothing to run under yet: all eight warps
-        row_stats(Item(a, it), stat, tid, kWorkers);
-        tc::bar_sync(1, kWorkers);
-      }
-      ok = ok && tc::mbar_wait(&bar_t[n & 1], (n >> 1) & 1, a.status);
       for (int kt = 0; kt < nq; ++kt, ++c) {
         for (int qt = kt; qt < nq; ++qt, ++p) {
           const bool diag = qt == kt;
-          const float2 st = rs[qt * kTile];
+          if (kt == 0) {
+            ok = ok && tc::mbar_wait(&bar_t[qt], (tph >> qt) & 1, a.status);
+            tph ^= 1u << qt;
+          }
+          const float2 st = stat[qt * kTile + r];
           ok = ok && tc::mbar_wait(bar_s, p & 1, a.status);
           tc::fence_after_sync();
           uint32_t s[2][32], dp[2][32];
@@ -389,10 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_proxy_async_smem();
         tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) {
-          tc::mbar_arrive(&bar_e[c & 1]);
-          if (kt + 1 == nq) tc::mbar_arrive(&bar_d[n & 1]);
-        }
+        if (lane == 0) tc::mbar_arrive(&bar_e[c & 1]);
       }
     }
   }
@@ -424,19 +456,17 @@ template <int DH>
 cudaError_t bwd_blk(const Launch& lc, const AttnBwdArgs& ab) {
   const AttnArgs& f = ab.f;
   const int D = f.H * DH;
-  CUtensorMap m[7];
+  CUtensorMap m[8];
   if (!blk_map<DH>(&m[0], f.Q, f.ld_qkv, D, f.T, f.B) ||
       !blk_map<DH>(&m[1], f.K, f.ld_qkv, D, f.T, f.B) ||
       !blk_map<DH>(&m[2], f.V, f.ld_qkv, D, f.T, f.B) ||
       !blk_map<DH>(&m[3], ab.dO, f.ld_o, D, f.T, f.B) ||
       !blk_map<DH>(&m[4], ab.dQ, ab.ld_dqkv, D, f.T, f.B) ||
       !blk_map<DH>(&m[5], ab.dK, ab.ld_dqkv, D, f.T, f.B) ||
-      !blk_map<DH>(&m[6], ab.dV, ab.ld_dqkv, D, f.T, f.B))
+      !blk_map<DH>(&m[6], ab.dV, ab.ld_dqkv, D, f.T, f.B) ||
+      !blk_map<DH>(&m[7], f.O, f.ld_o, D, f.T, f.B))
     return cudaErrorInvalidValue;
   BlkArgs a;
-  a.O = (const bf16*)f.O;
-  a.dO = (const bf16*)ab.dO;
-  a.ld_o = f.ld_o;
   a.lse = f.lse;
   a.Drow = ab.Drow;
   a.T = f.T;
@@ -455,7 +485,7 @@ cudaError_t bwd_blk(const Launch& lc, const AttnBwdArgs& ab) {
   if (cudaError_t e = smem_opt_in(kern, most, &opted); e != cudaSuccess) return e;
   cudaError_t e = launch_k(kern, dim3(a.total < sm_count() ? a.total : sm_count()), dim3(kThreads),
                            blk_smem<DH>(a.m), lc.stream, m[0], m[1], m[2], m[3], m[4], m[5], m[6],
-                           a);
+                           m[7], a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 }  // namespace
