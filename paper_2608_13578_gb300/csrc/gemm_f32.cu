@@ -5,10 +5,11 @@
 // two values the six of 2^-16 and above are formed, h h, h m, m h, m m, h l and
 // l h; each is exact in fp32.  The dropped ones are below 2^-24 of the product.
 // The tensor core's own accumulation is the weak point (its adds do not round
-// to nearest), so no h h accumulator lives longer than one 64-deep K slice: h h goes
-// to one TMEM accumulator, which the epilogue warps add to fp32 sums in registers
-// after every slice, and the five small products, 2^-8 of it and less, to a second,
-// added every kGroup slices.
+// to nearest), so no accumulator lives longer than one 64-deep K slice: h h goes
+// to one TMEM accumulator and the five small products to a second, and the
+// epilogue warps add both to fp32 sums in registers after every slice.  (The small
+// products left in their accumulator for eight slices: 8192 x 1536 x 512 84 us instead
+// of 88, but a relative error of 13.1e-8 instead of 12.7e-8 at K = 2048.)
 // Against float64 (N(0,1) rows x N(0,1/K) weights) the relative 2-norm error
 // is no larger than that of the CUDA-core kernel with its chain of K fused
 // multiply-adds (tests/test_gpu_gemm_f32.py compares the two).
@@ -21,7 +22,7 @@
 // shared memory with TMA; warp 8 also issues the MMAs, one slice ahead of its
 // draining (a warp of its own for that would cost every thread a quarter of its
 // registers, and a loader that issues them holds up all the splitting).
-// 8192 x 1536 x 512 takes 84 us (153 TFLOP/s of fp32 products; 122 us with a loader
+// 8192 x 1536 x 512 takes 88 us (146 TFLOP/s of fp32 products; 122 us with a loader
 // warp issuing the MMAs, 96 with their branch taken by lane number, see elect_one),
 // 512 x 1536 x 8192 in 3 splits 73 us (177); the CUDA-core kernel took 497 and 749
 // us.  A 64-deep slice of a 128 x 128 tile is 1536 cycles of tensor work and 2300 of
@@ -47,12 +48,6 @@ constexpr int kBM = 128, kBK = 64;
 constexpr int kLoadThreads = 256;
 constexpr int kThreads = 512;
 constexpr int kStages = 2;
-// Slices whose small products share an accumulator: draining it with every slice took
-// 88 us for 8192 x 1536 x 512, one drain in eight 84.  Relative 2-norm error against
-// float64 at K = 64, 512, 2048, 8192: 7.1, 9.0, 13.1, 22.8 e-8 (7.1, 9.0, 12.7, 21.7 with
-// every slice drained); an fp32 training step's largest error is 4.7e-7, with the
-// CUDA-core kernel 1.4e-6.
-constexpr int kGroup = 8;
 
 template <int BN>
 struct Cfg {
@@ -109,6 +104,17 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& 
   b -= __uint_as_float(h & 0xffff0000u);
   m = pack_bf16(a, b);
   l = pack_bf16(a - __uint_as_float(m << 16), b - __uint_as_float(m & 0xffff0000u));
+}
+
+// 16 columns of the warp's TMEM lane quarter, without waiting.
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
 }
 
 // The loader's share of a ROWS x 64 slice of one operand: units of eight
@@ -226,10 +232,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     ke = min(K, kb + kps * kBK);
   };
 
-  // slice `it`'s MMAs (one thread): h h into accumulator it & 1, the small products
-  // into accumulator g & 1, which is new where the slice opens a group
+  // slice `it`'s MMAs, into accumulator pair it & 1 (one thread)
   constexpr uint32_t idesc = tc::idesc_bf16(kBM, BN, A_MN ? 1 : 0, B_MN ? 1 : 0);
-  auto issue = [&](int it, int g, bool opens) {
+  auto issue = [&](int it) {
     const int s = it % kStages, acc = it & 1, use = it >> 1;
     if ((use > 0 && !tc::mbar_wait(&tempty[acc], (use - 1) & 1, status)) ||
         !tc::mbar_wait(&full[s], (it / kStages) & 1, status))
@@ -238,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t sa = tc::smem_u32(smem + s * C::STAGE);
     const uint64_t ad = tc::sdesc(sa, A_MN ? 8192 : 16, 1024),
                    bd = tc::sdesc(sa + 3 * C::A_PART, B_MN ? 8192 : 16, 1024);
-    const uint32_t d = tmem + (uint32_t)(acc * BN), d1 = tmem + (uint32_t)((2 + (g & 1)) * BN);
+    const uint32_t d = tmem + (uint32_t)(acc * 2 * BN);
     auto product = [&](int pa, int pb, uint32_t dst, bool first) {
 #pragma unroll
       for (int kk = 0; kk < kBK / 16; ++kk) {
@@ -248,11 +253,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     };
     product(0, 0, d, true);       // h h
-    product(0, 2, d1, opens);     // the small products, smallest first
-    product(2, 0, d1, false);
-    product(1, 1, d1, false);
-    product(0, 1, d1, false);
-    product(1, 0, d1, false);
+    product(0, 2, d + BN, true);  // the small products, smallest first
+    product(2, 0, d + BN, false);
+    product(1, 1, d + BN, false);
+    product(0, 1, d + BN, false);
+    product(1, 0, d + BN, false);
     tc::mma_commit(&empty[s]);
     tc::mma_commit(&tfull[acc]);
     return true;
@@ -305,31 +310,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3, c_beg = ((warp - 8) >> 2) * NC;
     uint8_t* sbuf = smem + C::OUT_OFF + (warp - 8) * 4096;
     const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c_beg;
-    int it = 0, g = 0;
-    // warp 8 also issues the MMAs, a slice ahead of its draining: the slice to issue,
-    // its tile, that tile's slices, its place among them, its group
-    int ii = 0, ti = blockIdx.x, ni = 0, si = 0, gi = -1;
-    auto slices_of = [&](int tile) {
-      if (tile >= n_tiles) return 0;
-      int m0, n0, z, kb, ke;
-      tile_at(tile, m0, n0, z, kb, ke);
-      return (ke - kb + kBK - 1) / kBK;
-    };
-    auto issue_next = [&]() {
-      while (si == ni && ti < n_tiles) {  // the next tile that has any slices
-        ni = slices_of(ti);
-        ti += gridDim.x;
-        si = 0;
+    int it = 0, slices = 0;  // warp 8 also issues the MMAs, a slice ahead of its draining
+    if (warp == 8)
+      for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        int m0, n0, z, kb, ke;
+        tile_at(tile, m0, n0, z, kb, ke);
+        slices += (ke - kb + kBK - 1) / kBK;
       }
-      if (si == ni) return;
-      const bool opens = si % kGroup == 0;
-      gi += opens;
-      if (tc::elect_one()) issue(ii, gi, opens);
-      __syncwarp();
-      ++ii;
-      ++si;
-    };
-    if (warp == 8) issue_next();
+    if (slices > 0 && tc::elect_one()) issue(0);
+    __syncwarp();
     bool ok = true;
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       int m0, n0, z, kb, ke;
@@ -337,31 +326,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       float acc[NC];
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[c] = 0.f;
-      int s = 0;
       for (int k = kb; k < ke; k += kBK, ++it) {
         const int ab = it & 1, use = it >> 1;
-        if (warp == 8) issue_next();
+        if (it + 1 < slices && tc::elect_one()) issue(it + 1);
+        __syncwarp();
         ok = tc::mbar_wait(&tfull[ab], use & 1, status) && ok;
         tc::fence_after_sync();
 #pragma unroll
-        for (int c = 0; c < NC; c += 32) {
-          uint32_t x[32];
-          tc::tmem_ld32_issue(trow + (uint32_t)(ab * BN + c), x);
+        for (int c = 0; c < NC; c += 16) {
+          uint32_t x[16], y[16];
+          tmem_ld16_issue(trow + (uint32_t)(ab * 2 * BN + c), x);
+          tmem_ld16_issue(trow + (uint32_t)(ab * 2 * BN + BN + c), y);
           tc::tmem_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) acc[c + j] += __uint_as_float(x[j]);
-        }
-        if (++s == kGroup || k + kBK >= ke) {  // the group's last slice
-#pragma unroll
-          for (int c = 0; c < NC; c += 32) {
-            uint32_t x[32];
-            tc::tmem_ld32_issue(trow + (uint32_t)((2 + (g & 1)) * BN + c), x);
-            tc::tmem_wait();
-#pragma unroll
-            for (int j = 0; j < 32; ++j) acc[c + j] += __uint_as_float(x[j]);
-          }
-          s = 0;
-          ++g;
+          for (int j = 0; j < 16; ++j)
+            acc[c + j] += __uint_as_float(x[j]) + __uint_as_float(y[j]);
         }
         tc::fence_before_sync();
         __syncwarp();
