@@ -29,7 +29,7 @@
 // of 96 L48 1161 -> 45 us.
 //
 // A masked key's weight is exactly 0, but 0 x inf = NaN in the products: a row
-// whose result is not finite is recomputed from its visible keys alone
+// whose result is not finite is formed again from its visible keys alone
 // (attn_slow.cuh).
 #include "attn_common.cuh"
 #include "attn_slow.cuh"
@@ -164,27 +164,55 @@ __device__ __forceinline__ bool aligned_smem(const uint8_t* smem, unsigned* stat
   return false;
 }
 
-// Staged rows recomputed from their visible keys / queries alone: 16-byte units
-// u0 .. u0+nu-1 of row r of the staging tile.
-__device__ __forceinline__ void put_staged(uint8_t* tile, int r, int u, const float* v) {
-  *reinterpret_cast<uint4*>(tile + (u >> 3) * kChunk + tc::sw128_offset(r, u & 7)) = pack8(v);
+// The 16-byte units (eight columns) of the thread's half row that are not finite.
+template <int OC>
+__device__ __forceinline__ unsigned bad_units(const float* v, int c0, int dh) {
+  unsigned bad = 0u;
+#pragma unroll
+  for (int c = 0; c < OC; ++c)
+    if (c0 + c < dh && !is_finite(v[c])) bad |= 1u << (c / 8);
+  return bad;
 }
-__device__ __noinline__ void restage_dq(const GenArgs& a, int b, int h, int t, uint8_t* tile, int r,
-                                        int u0, int nu) {
-  for (int u = u0; u < u0 + nu && 8 * u < a.x.dh; ++u) {
-    float v[8];
-    slow_dq<8>(a.x, b, h, t, 8 * u, v);
-    put_staged(tile, r, u, v);
+// Those of the CTA's rows formed again, row by row, in the staging tiles (bad: of row r
+// from unit u0 on; sm: free shared memory).
+__device__ __forceinline__ void put_units(uint8_t* tile, int r, const SlowRow& row, unsigned units,
+                                          int dh) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int c = (threadIdx.x & 31) + 32 * i, u = c / 8;
+    if (c < dh && (units >> u & 1u))
+      *reinterpret_cast<bf16*>(tile + (u >> 3) * kChunk + tc::sw128_offset(r, u & 7) + 2 * (c & 7)) =
+          from_f<bf16>(row.v[i]);
   }
 }
-__device__ __noinline__ void restage_dkv(const GenArgs& a, int b, int h, int j, uint8_t* tk,
-                                         uint8_t* tv, int r, int u0, int nu) {
-  for (int u = u0; u < u0 + nu && 8 * u < a.x.dh; ++u) {
-    float dk[8], dv[8];
-    slow_dkv<8>(a.x, b, h, j, 8 * u, dk, dv);
-    put_staged(tk, r, u, dk);
-    put_staged(tv, r, u, dv);
-  }
+__device__ __noinline__ void restage_dq(const GenArgs& a, int b, int h, int t0, uint8_t* tile, int r,
+                                        int u0, unsigned bad, uint8_t* sm) {
+  slow_rows<kTile>(reinterpret_cast<float*>(sm), [&](auto set) {
+    for (int u = 0; u < 8; ++u)
+      if (bad >> u & 1u) set(r, u0 + u);
+  }, [&](int n, unsigned units, float* w) {
+    SlowRow dq;
+    slow_dq(a.x, b, h, t0 + n, w, dq);
+    put_units(tile, n, dq, units, a.x.dh);
+  });
+}
+__device__ __noinline__ void restage_dkv(const GenArgs& a, int b, int h, int t0, uint8_t* tk,
+                                         uint8_t* tv, int r, int u0, unsigned badk, unsigned badv,
+                                         uint8_t* sm) {
+  slow_rows<2 * kTile>(reinterpret_cast<float*>(sm), [&](auto set) {
+    for (int u = 0; u < 8; ++u) {
+      if (badk >> u & 1u) set(r, u0 + u);
+      if (badv >> u & 1u) set(kTile + r, u0 + u);
+    }
+  }, [&](int n, unsigned units, float* w) {
+    const int row = n & (kTile - 1);
+    SlowRow d;
+    if (n < kTile)
+      slow_dkv<false>(a.x, b, h, t0 + row, w, d);
+    else
+      slow_dkv<true>(a.x, b, h, t0 + row, w, d);
+    put_units(n < kTile ? tk : tv, row, d, units, a.x.dh);
+  });
 }
 }  // namespace
 
@@ -327,12 +355,9 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     tc::fence_after_sync();
   }
 
-  bool fin = true;
-#pragma unroll
-  for (int c = 0; c < OC; ++c)
-    if (hf * OC + c < a.x.dh) fin = fin && is_finite(acc[c]);
+  const unsigned bad = row_ok ? bad_units<OC>(acc, hf * OC, a.x.dh) : 0u;
   stage_half<NC>(sQ, r, hf, acc);
-  if (!fin && row_ok) restage_dq(a, b, h, tt.t0 + r, sQ, r, hf * OC / 8, OC / 8);
+  if (__syncthreads_or(bad)) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, bad, sSh);
   tc::fence_proxy_async_smem();
   __syncthreads();
   if (warp0 && tc::elect_one() && ok) {
@@ -527,22 +552,19 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   }
 
   // ---- rows of dV, dK (key r) and, FUSED, dQ (query r) through staging tiles
-  auto staged = [&](uint32_t col, uint8_t* tile) {  // true: the row is finite
+  auto staged = [&](uint32_t col, uint8_t* tile) {  // the row's units that are not finite
     float v[OC];
     tmem_half<NC>(trow + col + (uint32_t)(hf * OC), v);
-    bool fin = true;
-#pragma unroll
-    for (int c = 0; c < OC; ++c)
-      if (hf * OC + c < a.x.dh) fin = fin && is_finite(v[c]);
     stage_half<NC>(tile, r, hf, v);
-    return fin;
+    return r < tt.rows ? bad_units<OC>(v, hf * OC, a.x.dh) : 0u;
   };
-  const bool fv = staged(kDV, sdO), fk = staged(kDK, sK);
-  if (!(fv && fk) && r < tt.rows)
-    restage_dkv(a, b, h, tt.t0 + r, sK, sdO, r, hf * OC / 8, OC / 8);
-  __syncwarp();
-  if (FUSED && !staged(kDQ, sQ) && r < tt.rows)
-    restage_dq(a, b, h, tt.t0 + r, sQ, r, hf * OC / 8, OC / 8);
+  const unsigned badv = staged(kDV, sdO), badk = staged(kDK, sK),
+                 badq = FUSED ? staged(kDQ, sQ) : 0u;
+  if (__syncthreads_or(badk | badv | badq)) {
+    restage_dkv(a, b, h, tt.t0, sK, sdO, r, hf * OC / 8, badk, badv, sPh);
+    __syncthreads();
+    if (FUSED) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, badq, sPh);
+  }
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
   __syncthreads();
@@ -579,10 +601,10 @@ constexpr int kExtra = 64;  // beside the tiles: barriers and the TMEM slot
 GenArgs gen_args(const Launch& lc, const AttnBwdArgs& ab) {
   const AttnArgs& a = ab.f;
   GenArgs g;
-  g.x = AttnPtrs<bf16>{(const bf16*)a.Q, (const bf16*)a.K,  (const bf16*)a.V, (const bf16*)a.O,
-                       (const bf16*)ab.dO, a.ld_qkv,          a.ld_o,           a.lse,
-                       a.T,              a.H,               a.dh,             a.L,
-                       1.0f / sqrtf((float)a.dh)};
+  g.x = AttnPtrs<bf16>{(const bf16*)a.Q, (const bf16*)a.K, (const bf16*)a.V, (const bf16*)a.O,
+                       (const bf16*)ab.dO, a.ld_qkv, a.ld_o, a.lse,
+                       a.L > kTile ? ab.Drow : nullptr, a.T, a.H, a.dh, a.L,
+                       1.0f / sqrtf((float)a.dh), 1};
   g.Drow = ab.Drow;
   g.rows = a.L <= kTile ? (kTile / a.L) * a.L : kTile;
   g.tpb = a.L <= kTile ? 1 : (a.L + kTile - 1) / kTile;

@@ -313,6 +313,62 @@ __device__ __forceinline__ int block_end(int r, int L) {
 }
 }  // namespace
 
+namespace {
+// The groups of four columns that came out non-finite, formed again row by row; bit
+// i * CB + m of bad: the thread's row i, column block m.
+template <int C4, int CB, class S>
+__device__ __forceinline__ void mark_bad(S&& set, int row0, unsigned bad) {
+  using C = Cols<C4, CB>;
+  for (int n = 0; n < C::RT * CB; ++n)
+    if (bad >> n & 1u) set(row0 + C::row() + n / CB, C::col() / 4 + 16 * (n % CB));
+}
+template <class E>
+__device__ __forceinline__ void put_groups(E* p, const SlowRow& r, unsigned groups, int dh) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int c = (threadIdx.x & 31) + 32 * i;
+    if (c < dh && (groups >> (c / 4) & 1u)) p[c] = from_f<E>(r.v[i]);
+  }
+}
+template <class E, int C4, int CB>
+__device__ __noinline__ void redo_o(const SimtArgs<E>& a, const TileAt& tt, float* sm, unsigned bad) {
+  E* out = a.Out + ((long)tt.b * a.x.T + tt.t0) * a.x.ld_o + tt.h * a.x.dh;
+  slow_rows<kTile>(sm, [&](auto set) { mark_bad<C4, CB>(set, 0, bad); },
+                   [&](int r, unsigned groups, float* w) {
+    SlowRow o;
+    slow_o(a.x, tt.b, tt.h, tt.t0 + r, w, o);
+    put_groups(out + r * a.x.ld_o, o, groups, a.x.dh);
+  });
+}
+template <class E, int C4, int CB>
+__device__ __noinline__ void redo_dq(const SimtArgs<E>& a, const TileAt& tt, float* sm, unsigned bad) {
+  E* out = a.dQ + ((long)tt.b * a.x.T + tt.t0) * a.ld_d + tt.h * a.x.dh;
+  slow_rows<kTile>(sm, [&](auto set) { mark_bad<C4, CB>(set, 0, bad); },
+                   [&](int r, unsigned groups, float* w) {
+    SlowRow dq;
+    slow_dq(a.x, tt.b, tt.h, tt.t0 + r, w, dq);
+    put_groups(out + r * a.ld_d, dq, groups, a.x.dh);
+  });
+}
+template <class E, int C4, int CB>
+__device__ __noinline__ void redo_dkv(const SimtArgs<E>& a, const TileAt& tt, float* sm,
+                                      unsigned badk, unsigned badv) {
+  const long o = ((long)tt.b * a.x.T + tt.t0) * a.ld_d + tt.h * a.x.dh;
+  slow_rows<2 * kTile>(sm, [&](auto set) {
+    mark_bad<C4, CB>(set, 0, badk);
+    mark_bad<C4, CB>(set, kTile, badv);
+  }, [&](int n, unsigned groups, float* w) {
+    const int r = n & (kTile - 1);
+    SlowRow d;
+    if (n < kTile)
+      slow_dkv<false>(a.x, tt.b, tt.h, tt.t0 + r, w, d);
+    else
+      slow_dkv<true>(a.x, tt.b, tt.h, tt.t0 + r, w, d);
+    put_groups((n < kTile ? a.dK : a.dV) + o + r * a.ld_d, d, groups, a.x.dh);
+  });
+}
+}  // namespace
+
 // O[t] = sum_j softmax_j(q_t . k_j * scale) v_j over keys j in [blockstart(t), t].
 //
 // The arithmetic and its order are those of one query at a time -- a score is
@@ -446,6 +502,7 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 3 : 2)
     a.lse[((long)b * a.x.H + h) * a.x.T + tt.t0 + r] = m + logf(inv[r]);
   }
   const int c = C::col();
+  unsigned bad = 0u;
 #pragma unroll
   for (int i = 0; i < C::RT; ++i) {
     const int r = C::row() + i, t = tt.t0 + r;
@@ -457,10 +514,11 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 3 : 2)
         float* v = acc[i][m];
 #pragma unroll
         for (int e = 0; e < 4; ++e) v[e] *= in;
-        if (!finite4(v)) slow_o<4>(a.x, b, h, t, c + 64 * m, v);
+        if (!finite4(v)) bad |= 1u << (i * CB + m);
         put4(a.Out + (row0 + t) * a.x.ld_o + c0 + c + 64 * m, v, true);
       }
   }
+  if (__syncthreads_or(bad)) redo_o<E, C4, CB>(a, tt, sm, bad);
 }
 
 namespace {
@@ -530,11 +588,13 @@ __device__ __forceinline__ void rows_lse(const SimtArgs<E>& a, int b, int h, int
   for (int i = 0; i < 4; ++i)
     v[i] = 4 * ty + i < rows ? src[((long)b * a.x.H + h) * a.x.T + t0 + 4 * ty + i] : 0.f;
 }
+// Stores the thread's dQ; the groups that are not finite (as `bad` above).
 template <class E, int C4, int CB>
-__device__ __forceinline__ void store_dq(const SimtArgs<E>& a, const TileAt& tt, int b, int h,
-                                         float (*acc)[CB][4]) {
+__device__ __forceinline__ unsigned store_dq(const SimtArgs<E>& a, const TileAt& tt, int b, int h,
+                                             float (*acc)[CB][4]) {
   using C = Cols<C4, CB>;
   const int c = C::col();
+  unsigned bad = 0u;
 #pragma unroll
   for (int i = 0; i < C::RT; ++i) {
     const int r = C::row() + i, t = tt.t0 + r;
@@ -542,10 +602,11 @@ __device__ __forceinline__ void store_dq(const SimtArgs<E>& a, const TileAt& tt,
 #pragma unroll
     for (int m = 0; m < CB; ++m)
       if (c + 64 * m < a.x.dh) {
-        if (!finite4(acc[i][m])) slow_dq<4>(a.x, b, h, t, c + 64 * m, acc[i][m]);
+        if (!finite4(acc[i][m])) bad |= 1u << (i * CB + m);
         put4(a.dQ + ((long)b * a.x.T + t) * a.ld_d + h * a.x.dh + c + 64 * m, acc[i][m], a.vec);
       }
   }
+  return bad;
 }
 }  // namespace
 
@@ -590,7 +651,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, 0,
                        C::row() >= tt.rows ? 0 : diag ? min(C::row() + C::RT, nk) : kTile, 0, acc);
   }
-  store_dq<E, C4, CB>(a, tt, b, h, acc);
+  const unsigned bad = store_dq<E, C4, CB>(a, tt, b, h, acc);
+  if (__syncthreads_or(bad)) redo_dq<E, C4, CB>(a, tt, sm, bad);
 }
 
 // Per key tile: dV_j = sum_t P_tj dO_t, dK_j = scale * sum_t P_tj (dO_t . v_j - Drow_t) q_t
@@ -640,6 +702,7 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     cols_times<C4, CB>(Ss, Qs, ldh, dh, lo, hi, dk);
   }
   const int c = C::col();
+  unsigned badk = 0u, badv = 0u;
 #pragma unroll
   for (int i = 0; i < C::RT; ++i) {
     const int r = C::row() + i, t = tt.t0 + r;
@@ -647,8 +710,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
 #pragma unroll
     for (int m = 0; m < CB; ++m)
       if (c + 64 * m < dh) {
-        if (!(finite4(dk[i][m]) && finite4(dv[i][m])))
-          slow_dkv<4>(a.x, b, h, t, c + 64 * m, dk[i][m], dv[i][m]);
+        if (!finite4(dk[i][m])) badk |= 1u << (i * CB + m);
+        if (!finite4(dv[i][m])) badv |= 1u << (i * CB + m);
         const long o = (row0 + t) * a.ld_d + c0 + c + 64 * m;
         put4(a.dV + o, dv[i][m], a.vec);
         put4(a.dK + o, dk[i][m], a.vec);
@@ -659,8 +722,10 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     zero<C::RT, CB>(dq);
     rows_times<C4, CB>(Ss, kPld, Ks, ldh, dh, block_row(C::row(), a.x.L),
                        C::row() >= tt.rows ? 0 : min(C::row() + C::RT, tt.rows), 0, dq);
-    store_dq<E, C4, CB>(a, tt, b, h, dq);
+    const unsigned badq = store_dq<E, C4, CB>(a, tt, b, h, dq);
+    if (__syncthreads_or(badq)) redo_dq<E, C4, CB>(a, tt, sm, badq);
   }
+  if (__syncthreads_or(badk | badv)) redo_dkv<E, C4, CB>(a, tt, sm, badk, badv);
 }
 
 namespace {
@@ -668,8 +733,9 @@ template <class E>
 SimtArgs<E> simt_args(const AttnArgs& f, const AttnBwdArgs* ab) {
   SimtArgs<E> a;
   a.x = AttnPtrs<E>{(const E*)f.Q, (const E*)f.K, (const E*)f.V, (const E*)f.O,
-                    ab ? (const E*)ab->dO : nullptr, f.ld_qkv, f.ld_o, f.lse, f.T, f.H, f.dh, f.L,
-                    1.0f / sqrtf((float)f.dh)};
+                    ab ? (const E*)ab->dO : nullptr, f.ld_qkv, f.ld_o, f.lse,
+                    ab && f.L > kTile ? ab->Drow : nullptr, f.T, f.H, f.dh, f.L,
+                    1.0f / sqrtf((float)f.dh), f.ld_qkv % 8 == 0};
   a.Out = (E*)f.O;
   a.dQ = ab ? (E*)ab->dQ : nullptr;
   a.dK = ab ? (E*)ab->dK : nullptr;

@@ -4,7 +4,12 @@ some, and that no bounded wait runs out over it.
 Limits.  A NaN makes the affected outputs be formed again from the operands: a walk
 over K per row and column of a 32 x 32 run, at most a few times the product itself (its
 three-part split reads each operand once per output tile).  40 times the finite call
-leaves room for the timer; a chain of K terms per output took 10^3 times and more."""
+leaves room for the timer; a chain of K terms per output took 10^3 times and more.  An
+attention row of NaN is known from its first keys: 8 times the finite call.  One token
+that is not finite makes up to 128 rows, 16 a warp, walk 1024 keys, 32 at a time, with
+up to four dot products of 128 each: 16 x 32 x (4 x 128 x 8 + 1500) cycles, 1.5 ms, in
+each of two kernels, against 0.1 ms for the fastest finite backward; 60 times is the
+limit, twice that (a thread per row and group of columns took 150 to 20000 times)."""
 
 import pytest
 import torch
@@ -67,6 +72,38 @@ def test_product_with_nan_costs_a_few_products(C, lay, M, N, K, where):
     C.bcmt_device_status()
     assert torch.equal(torch.isnan(out), bad)
     assert nan <= 40 * finite, (nan, finite)
+
+
+@pytest.mark.parametrize("what,limit", [("all", 8), ("key", 60), ("value", 60)])
+@pytest.mark.parametrize("dtype,impl", [("fp32", 0), ("bf16", 0), ("bf16", 3)])
+def test_non_finite_attention_costs_a_few_calls(C, dtype, impl, what, limit):
+    B, T, H, dh, L = 2, 2048, 4, 128, 1024
+    D, dt = H * dh, torch.float32 if dtype == "fp32" else torch.bfloat16
+    p = C.make_params(B, T, D, H, L, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    ins = [torch.randn(B, T, D, generator=gen, device="cuda").to(dt) for _ in range(4)]
+    o, lse = torch.empty_like(ins[0]), torch.empty(B, H, T, device="cuda")
+    drow, g = torch.empty_like(lse), [torch.empty_like(ins[0]) for _ in range(3)]
+
+    def both(q, k, v, dO):
+        return (_ms(lambda: C.bcmt_test_attn(0, 0, p, q, k, v, D, o, lse)),
+                _ms(lambda: C.bcmt_test_attn(impl, 1, p, q, k, v, D, o, lse, dO, drow, *g, D)))
+
+    finite = both(*ins)
+    if what == "all":
+        ins = [torch.full_like(x, NAN) for x in ins]
+    else:  # a token near the end of the first block
+        ins[1 if what == "key" else 2][0, L - 2] = NAN if what == "key" else INF
+    bad = both(*ins)
+    C.bcmt_device_status()
+    if what == "all":
+        assert all(torch.isnan(x).all() for x in (o, lse, *g))
+    else:  # the forward's rows that see it and no others
+        rows = torch.zeros(B, T, dtype=torch.bool, device="cuda")
+        rows[0, L - 2:L] = True
+        assert torch.equal(torch.isfinite(o).all(-1), ~rows)
+        assert torch.equal(torch.isfinite(g[0]).all(-1), ~rows)
+    assert bad[0] <= limit * finite[0] and bad[1] <= limit * finite[1], (bad, finite)
 
 
 def test_product_with_infinities(C):
