@@ -24,6 +24,11 @@ extern "C" {
  * choice (the K-split layouts differ): query them after calling it. */
 int bcmt_test_set_tensor_cores(int gemm_on, int attn_on);
 
+/* on = 0: bcmt_forward / bcmt_backward keep every launch on the caller's stream from
+ * now on in this process, as they do where the side streams cannot be created; 1 (the
+ * default): the side streams are used. */
+void bcmt_test_set_side_streams(int on);
+
 /* C[M,N] = A[M,K] B[K,N] with fp32 accumulation, element (m,k) of A at
  * A[m*sam + k*sak] and (k,n) of B at B[k*sbk + n*sbn] (elements, not bytes);
  * C row-major with leading dimension ldc, of type dtype_out.  impl: 0 SIMT,

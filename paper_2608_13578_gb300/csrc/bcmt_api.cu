@@ -164,6 +164,7 @@ struct Fork {
 // Tensor-core paths of the layer (switchable only through bcmt_testing.h).
 bool g_use_tc_gemm = true;
 bool g_use_tc_attn = true;
+bool g_use_side_streams = true;  // switchable likewise
 
 // ------------------------------------------------------------------ profiling
 struct ProfRec {
@@ -651,7 +652,7 @@ bcmt_status bcmt_forward(const bcmt_params* p, const void* x, const void* q, con
   const bool profiling = (p->flags & BCMT_FLAG_PROFILE) != 0;
   // The memory stage runs on the side stream beside the gate GEMM (one
   // stream while profiling).
-  std::unique_ptr<Fork> fork_holder(new Fork(profiling ? nullptr : side_stream(), s));
+  std::unique_ptr<Fork> fork_holder(new Fork(profiling || !g_use_side_streams ? nullptr : side_stream(), s));
   Fork& fork = *fork_holder;
   Launch lc{fork.main(), sp};
   Prof pr{profiling, fork.main()};
@@ -843,7 +844,7 @@ bcmt_status bcmt_backward(const bcmt_params* p, const void* dy, const void* x_or
   const bool profiling = (p->flags & BCMT_FLAG_PROFILE) != 0;
   // Weight gradients go to the side stream (kept on one stream while
   // profiling, so every kernel is timed alone).
-  std::unique_ptr<Fork> fork_holder(new Fork(profiling ? nullptr : side_stream(), s));
+  std::unique_ptr<Fork> fork_holder(new Fork(profiling || !g_use_side_streams ? nullptr : side_stream(), s));
   Fork& fork = *fork_holder;
   Launch lc{fork.main(), sp};
   Prof pr{profiling, fork.main()};
@@ -1236,6 +1237,8 @@ int bcmt_test_set_tensor_cores(int gemm_on, int attn_on) {
   g_use_tc_attn = attn_on != 0;
   return (gemm_tc_available() ? 1 : 0) | (attn_tc_supported(1, 64, 64) ? 2 : 0);
 }
+
+void bcmt_test_set_side_streams(int on) { g_use_side_streams = on != 0; }
 
 int bcmt_test_wait_expiry(long long cycles, void* stream) {
   if (cycles < 1 || cycles > tc::kWaitCycles) {

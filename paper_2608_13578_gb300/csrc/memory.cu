@@ -503,11 +503,22 @@ __global__ void __launch_bounds__(kThreads, 2)
   const bf16* Hb = Hm + rowbase * D;
   bf16* dHb = dH + rowbase * D;
   const bf16* dYb = dY + rowbase * D;
+  pdl_enter();
+  dYb = after_wait(dYb);
+  Hb = after_wait(Hb);
+  dHb = after_wait(dHb);
+  alpha = after_wait(alpha);
+  Sb = after_wait(Sb);
+  dS = after_wait(dS);
+  if (n <= 0) {  // a ragged last block's empty chunk: zero partials of dW_p
+    for (int k = threadIdx.x; k < D; k += kThreads) dwp_part[prow * D + k] = 0.f;
+    return;
+  }
   // dY goes straight to shared memory (cp.async: no registers held while it
-  // is in flight), each thread's own pieces, read back by the same thread.
-  // dY was read by the call's first kernel, whose completion the memory
-  // gradient's stream (joined just before this launch) has waited for, so its
-  // copies go out before the wait for the previous kernel.
+  // is in flight), each thread's own pieces, read back by the same thread.  (Only
+  // after the wait: where the layer has no side streams the launches since the
+  // call's first kernel are a chain of early starts, and the layer above may
+  // still be writing dY.)
   extern __shared__ __align__(16) uint8_t ys_raw[];  // [8 RW rows][KC * 256] bf16
   bf16* ys = reinterpret_cast<bf16*>(ys_raw);
 #pragma unroll
@@ -520,16 +531,6 @@ __global__ void __launch_bounds__(kThreads, 2)
                    dYb + (long)(warp + 8 * u) * D + k);
     }
   cp_async_commit();
-  pdl_enter();
-  Hb = after_wait(Hb);
-  dHb = after_wait(dHb);
-  alpha = after_wait(alpha);
-  Sb = after_wait(Sb);
-  dS = after_wait(dS);
-  if (n <= 0) {  // a ragged last block's empty chunk: zero partials of dW_p
-    for (int k = threadIdx.x; k < D; k += kThreads) dwp_part[prow * D + k] = 0.f;
-    return;
-  }
   uint4 h[RW][KC], d[RW][KC];
 #pragma unroll
   for (int u = 0; u < RW; ++u)
@@ -1021,6 +1022,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   alpha = after_wait(alpha);
   Sb = after_wait(Sb);
   dS = after_wait(dS);
+  dY = after_wait(dY);
   dH = after_wait(dH);
   __shared__ __align__(16) float sm[ROWS + 8 + 8 * 260];
   // a ragged last block has fewer chunks than the grid's x extent: its empty
