@@ -118,7 +118,9 @@ def _ptr(t) -> Optional[int]:
     try:
         return t.data_ptr()
     except AttributeError:
-        return int(t)
+        if isinstance(t, int):
+            return t
+        raise
 
 
 def _current_stream() -> int:
