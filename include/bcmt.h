@@ -180,16 +180,12 @@ bcmt_status bcmt_decode_step(const bcmt_params* p, void* state, long pos, const 
  * (B, T, D, H, L, dtype; input_is_x and flags other than BCMT_FLAG_CHECK are
  * ignored).
  *
- * Its one scratch buffer (one fp32 per batch, head and token) is a device
- * array inside the library: 4 MiB, allocated on every GPU that loads the
- * library and held until the process exits.  B*H*T must not exceed 1048576;
- * larger shapes are rejected with BCMT_ERR_SHAPE before anything is launched.
- * The first call on a device looks up that array's device address (once per
- * device, with that device current); make that first call before any stream
- * capture.  All calls share the array and it keeps the last call's contents:
- * calls that overlap on the GPU (other streams, other threads) race on it, so
- * serialise them.  Nothing is allocated: no cudaMalloc, cudaFree or
- * allocating library routine is called. */
+ * It takes no scratch and the library keeps none for it: dO . O, which the layer's
+ * backward stores between its two kernels, is formed in each.  Calls share nothing, so
+ * they may overlap on other streams and threads and be captured.  B*H*T must not exceed
+ * 1048576; larger shapes are rejected with BCMT_ERR_SHAPE before anything is launched.
+ * Nothing is allocated: no cudaMalloc, cudaFree or allocating library routine is
+ * called. */
 bcmt_status bcmt_attention_backward_noalloc(const bcmt_params* p, const void* q, const void* k,
                                             const void* v, long ld, const void* o,
                                             const float* lse, const void* dO, void* dq, void* dk,

@@ -205,8 +205,8 @@ def bcmt_decode_step(p: bcmt_params, state, pos: int, x_t, w_qkv, w_o, w_p, w_m,
 
 def bcmt_attention_backward_noalloc(p: bcmt_params, q, k, v, ld, o, lse, dO, dq, dk, dv, ld_d,
                                     stream=None) -> None:
-    """Attention backward whose scratch is a device array inside the library
-    (for callers that cannot allocate device memory); see include/bcmt.h."""
+    """Attention backward without any scratch (for callers that cannot allocate
+    device memory); see include/bcmt.h."""
     _check(LIB.bcmt_attention_backward_noalloc(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(v), ld,
                                                _ptr(o), _ptr(lse), _ptr(dO), _ptr(dq), _ptr(dk),
                                                _ptr(dv), ld_d, _stream(stream)))

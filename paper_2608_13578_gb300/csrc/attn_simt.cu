@@ -23,7 +23,6 @@
 // bf16 forward 1997 and 126 us; B4 T1000 D768 h8 L48 bf16 forward 306 and 63 us.
 // Deterministic: every sum runs in a fixed order.
 #include <algorithm>
-#include <mutex>
 
 #include "attn_slow.cuh"
 #include "common.cuh"
@@ -525,15 +524,15 @@ namespace {
 // Drow of the thread's four rows, from the tensors: the 16 threads of a row
 // group share a row's columns.
 template <class E>
-__device__ __forceinline__ void drow4(const SimtArgs<E>& a, const TileAt& tt, int b, int h,
+__device__ __forceinline__ void drow4(const SimtArgs<E>& a, int b, int h, int t0, int rows,
                                       float* d) {
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = 4 * ty + i;
     float s = 0.f;
-    if (r < tt.rows) {
-      const long o = ((long)b * a.x.T + tt.t0 + r) * a.x.ld_o + h * a.x.dh;
+    if (r < rows) {
+      const long o = ((long)b * a.x.T + t0 + r) * a.x.ld_o + h * a.x.dh;
       for (int c = 4 * tx; c < a.x.dh; c += 64) {
         float u[4], v[4];
         load4(a.x.dO + o + c, u);
@@ -630,9 +629,9 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
   fill(Gs, ldh, a.x.dO + (row0 + tt.t0) * a.x.ld_o + c0, a.x.ld_o, tt.rows, dh, true);
   using C = Cols<C4, CB>;
   float drow[4], lse[4], acc[C::RT][CB][4];
-  drow4(a, tt, b, h, drow);
+  drow4(a, b, h, tt.t0, tt.rows, drow);
   rows_lse(a, b, h, tt.t0, tt.rows, a.lse, lse);
-  if (tx == 0) {
+  if (tx == 0 && a.Drow) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (4 * ty + i < tt.rows)
@@ -658,7 +657,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
 // Per key tile: dV_j = sum_t P_tj dO_t, dK_j = scale * sum_t P_tj (dO_t . v_j - Drow_t) q_t
 // over queries t in [j, blockend(j)), tile by tile.  FUSED (L <= 64, where the
 // tile is its own and only query tile): Drow is formed here and dQ joins, one
-// pass instead of two.
+// pass instead of two.  Without scratch for Drow (the allocation-free backward) each
+// query tile's is formed again here, by the same sums.
 template <class E, int C4, int CB, bool FUSED>
 __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     attn_bwd_kv_simt_kernel(const __grid_constant__ SimtArgs<E> a) {
@@ -687,8 +687,8 @@ __global__ void __launch_bounds__(kThreads, CB == 1 ? 2 : 1)
     fill(Qs, ldh, a.x.Q + (row0 + t0) * a.x.ld + c0, a.x.ld, rows, dh, a.vec);
     fill(Gs, ldh, a.x.dO + (row0 + t0) * a.x.ld_o + c0, a.x.ld_o, rows, dh, true);
     float drow[4], lse[4];
-    if (FUSED)
-      drow4(a, tt, b, h, drow);
+    if (FUSED || !a.Drow)
+      drow4(a, b, h, t0, rows, drow);
     else
       rows_lse(a, b, h, t0, rows, a.Drow, drow);
     rows_lse(a, b, h, t0, rows, a.lse, lse);
@@ -819,48 +819,6 @@ cudaError_t attn_fwd_simt(const Launch& lc, int dtype, const AttnArgs& a) {
 cudaError_t attn_bwd_simt(const Launch& lc, int dtype, const AttnBwdArgs& a) {
   if (a.f.dh > kMaxDh || a.f.L > kMaxL) return cudaErrorInvalidValue;
   return dtype == 0 ? bwd_typed<float>(lc, a) : bwd_typed<bf16>(lc, a);
-}
-
-// ------------------------------------------- allocation-free backward variant
-// The backward above needs one fp32 scratch value per (batch, head, token):
-// Drow = dO . O, written by the dQ kernel and read by the dK/dV kernel.  For
-// callers that cannot allocate device memory, this variant keeps that scratch
-// in a file-scope device array instead of caller memory.  It is allocated when
-// the library is loaded, once on every GPU that loads it, and held until the
-// process exits.  Every call shares it, so calls that overlap on the GPU (on
-// different streams, or from different threads) race on it.  The dQ kernel
-// writes every entry the dK/dV kernel reads, so nothing needs clearing between
-// calls even though the array keeps the last call's contents.
-static __device__ __align__(256) float g_noalloc_drow[kNoAllocDrowRows];
-
-namespace {
-constexpr int kMaxDevices = 64;
-std::mutex g_noalloc_mu;
-float* g_noalloc_ptr[kMaxDevices] = {};
-}  // namespace
-
-cudaError_t attn_bwd_simt_noalloc(const Launch& lc, int dtype, const AttnBwdArgs& a) {
-  if ((long long)a.f.B * a.f.H * a.f.T > kNoAllocDrowRows) return cudaErrorInvalidValue;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  float* drow = nullptr;
-  {
-    // Set-up, once per device with that device current: the array's name is
-    // only a host-side stand-in, so look up its device address.
-    std::lock_guard<std::mutex> lk(g_noalloc_mu);
-    if (!g_noalloc_ptr[dev]) {
-      void* p = nullptr;
-      e = cudaGetSymbolAddress(&p, g_noalloc_drow);
-      if (e != cudaSuccess) return e;
-      g_noalloc_ptr[dev] = static_cast<float*>(p);
-    }
-    drow = g_noalloc_ptr[dev];
-  }
-  AttnBwdArgs b = a;
-  b.Drow = drow;
-  return attn_bwd_simt(lc, dtype, b);
 }
 
 }  // namespace bcmt

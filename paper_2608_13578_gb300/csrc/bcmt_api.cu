@@ -1181,18 +1181,18 @@ bcmt_status bcmt_attention_backward_noalloc(const bcmt_params* p, const void* q,
   if (ld < g.D || ld_d < g.D)
     return fail(BCMT_ERR_ARG, "row strides ld = %ld and ld_d = %ld must be >= D = %d", ld, ld_d, g.D);
   const long long rows = (long long)g.B * g.H * g.T;
-  if (rows > kNoAllocDrowRows)
+  if (rows > kNoAllocRows)
     return fail(BCMT_ERR_SHAPE,
-                "B*H*T = %lld exceeds the %lld rows of the built-in scratch of "
-                "bcmt_attention_backward_noalloc",
-                rows, kNoAllocDrowRows);
+                "B*H*T = %lld exceeds the %lld rows that bcmt_attention_backward_noalloc, "
+                "which has no scratch, takes",
+                rows, kNoAllocRows);
   unsigned* sp = status_ptr();
   if (!sp) return fail(BCMT_ERR_CUDA, "no CUDA device / device status word unavailable");
   Launch lc{static_cast<cudaStream_t>(stream), sp};
   AttnBwdArgs ab{{q, k, v, ld, const_cast<void*>(o), g.D, const_cast<float*>(lse), g.B, g.T, g.H,
                   g.dh, g.L},
                  dO, nullptr, dq, dk, dv, ld_d};
-  cudaError_t e = attn_bwd_simt_noalloc(lc, g.dtype, ab);
+  cudaError_t e = attn_bwd_simt(lc, g.dtype, ab);  // (Drow null: it needs none)
   if (e != cudaSuccess) return cuda_fail(e, "allocation-free attention backward");
   return finish(p, lc.stream);
 }

@@ -182,11 +182,10 @@ struct AttnBwdArgs {
   void* dV;
   long ld_dqkv;
 };
+// Drow may be null: then each kernel forms what it needs of it.
 cudaError_t attn_bwd_simt(const Launch& lc, int dtype, const AttnBwdArgs& a);
-// The same backward with its Drow scratch in a static device array of
-// kNoAllocDrowRows floats instead of a.Drow; B*H*T must not exceed it.
-constexpr long long kNoAllocDrowRows = 1ll << 20;
-cudaError_t attn_bwd_simt_noalloc(const Launch& lc, int dtype, const AttnBwdArgs& a);
+// B*H*T of the allocation-free backward at most
+constexpr long long kNoAllocRows = 1ll << 20;
 
 cudaError_t attn_fwd_tc(const Launch& lc, const AttnArgs& a);
 cudaError_t attn_bwd_tc(const Launch& lc, const AttnBwdArgs& a);
