@@ -330,7 +330,7 @@ __device__ __forceinline__ void put_groups(E* p, const SlowRow& r, unsigned grou
   }
 }
 template <class E, int C4, int CB>
-__device__ __noinline__ void redo_o(const SimtArgs<E>& a, const TileAt& tt, float* sm, unsigned bad) {
+__device__ __noinline__ void redo_o(const SimtArgs<E>& a, TileAt tt, float* sm, unsigned bad) {
   E* out = a.Out + ((long)tt.b * a.x.T + tt.t0) * a.x.ld_o + tt.h * a.x.dh;
   slow_rows<kTile>(sm, [&](auto set) { mark_bad<C4, CB>(set, 0, bad); },
                    [&](int r, unsigned groups, float* w) {
@@ -340,7 +340,7 @@ __device__ __noinline__ void redo_o(const SimtArgs<E>& a, const TileAt& tt, floa
   });
 }
 template <class E, int C4, int CB>
-__device__ __noinline__ void redo_dq(const SimtArgs<E>& a, const TileAt& tt, float* sm, unsigned bad) {
+__device__ __noinline__ void redo_dq(const SimtArgs<E>& a, TileAt tt, float* sm, unsigned bad) {
   E* out = a.dQ + ((long)tt.b * a.x.T + tt.t0) * a.ld_d + tt.h * a.x.dh;
   slow_rows<kTile>(sm, [&](auto set) { mark_bad<C4, CB>(set, 0, bad); },
                    [&](int r, unsigned groups, float* w) {
@@ -350,7 +350,7 @@ __device__ __noinline__ void redo_dq(const SimtArgs<E>& a, const TileAt& tt, flo
   });
 }
 template <class E, int C4, int CB>
-__device__ __noinline__ void redo_dkv(const SimtArgs<E>& a, const TileAt& tt, float* sm,
+__device__ __noinline__ void redo_dkv(const SimtArgs<E>& a, TileAt tt, float* sm,
                                       unsigned badk, unsigned badv) {
   const long o = ((long)tt.b * a.x.T + tt.t0) * a.ld_d + tt.h * a.x.dh;
   slow_rows<2 * kTile>(sm, [&](auto set) {
