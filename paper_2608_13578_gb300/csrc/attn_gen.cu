@@ -13,20 +13,26 @@
 // Loads always bring 128 rows; the rows that belong to the next tile are
 // masked, and output boxes are as high as the tile has rows of its own.
 //
-// Precision.  The probabilities P and the score gradients dS are fp32 values;
-// as operands of the tensor-core products they enter as the sum of two bf16
-// numbers (hi = bf16(x), lo = bf16(x - hi): 16 significand bits), so that the
-// products see them to 2^-17 instead of bf16's 2^-9.  The other operands are
-// the bf16 tensors themselves.
+// Precision.  The probabilities P and the score gradients dS are fp32 values; as
+// operands of the tensor-core products they enter as the sum of three bf16 numbers,
+// which is exact (24 significand bits; below 2^-110 the last part underflows).  The other
+// operands are the bf16 tensors themselves.  Exponentials are ex2.approx of an argument
+// that is right to 2^-24 of its terms (Exp2; expf took 91 us where this takes 79).  Against
+// float64 on the same O, over 82 shapes (heads of 8 to 128, blocks of 16 to 1024), the
+// relative error of the bf16 gradients is the CUDA-core kernels' times 1.0000003 on average
+// (1.0000056 at most; times 0.9999986 against the gradients of the unrounded O), and 0.22 %
+// of the values round to another bf16 number than float64's (0.15 % there; with P and dS
+// as two parts each 0.63 %).
 //
 // Work split: 256 threads; warp w owns TMEM lane quarter w % 4 (thread = one
 // query row) and half w / 4 of the 128 key columns (of the dh output columns
 // in the epilogues).  What bounds it: the chain load -> S, dP -> P -> dV -> dS
 // -> dK, dQ of one CTA, several microseconds, covered by a second CTA per SM
-// where shared memory allows (heads up to 64).  Against the CUDA-core kernels
-// that served these shapes before (one warp per row, operands re-read from L2
-// per row): B4 T2048 D1024 heads of 128 L128 8230 -> 76 us, B4 T1000 D768 heads
-// of 96 L48 1161 -> 45 us.
+// where shared memory allows (heads up to 64, which then keep two parts in shared
+// memory at a time and the third in registers until the first two are multiplied).
+// Against the CUDA-core kernels that served these shapes before (one warp per row,
+// operands re-read from L2 per row): B4 T2048 D1024 heads of 128 L128 8230 -> 79 us,
+// B4 T1000 D768 heads of 96 L48 1161 -> 43 us (73 and 39 with two parts per value).
 //
 // A masked key's weight is exactly 0, but 0 x inf = NaN in the products: a row
 // whose result is not finite is formed again from its visible keys alone
@@ -45,7 +51,7 @@ namespace {
 constexpr int kTile = 128;
 constexpr int kThreads = 256;
 constexpr uint32_t kChunk = 16384;  // one 128-row x 64-column box
-constexpr uint32_t kP = 32768;      // one 128 x 128 bf16 operand (hi or lo part)
+constexpr uint32_t kP = 32768;      // one 128 x 128 bf16 operand (a part of P or dS)
 
 // What the kernels need beside their tensor maps.
 struct GenArgs {
@@ -56,21 +62,37 @@ struct GenArgs {
   unsigned* status;
 };
 
-// a, b as bf16 pairs hi + lo.
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  hi = pack2(a, b);
-  lo = pack2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+// a, b as bf16 pairs h + m + l, exactly.
+__device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+  h = pack2(a, b);
+  a -= __uint_as_float(h << 16);
+  b -= __uint_as_float(h & 0xffff0000u);
+  m = pack2(a, b);
+  l = pack2(a - __uint_as_float(m << 16), b - __uint_as_float(m & 0xffff0000u));
 }
-// Eight values into unit u of row r of the hi and lo operand tiles.
-__device__ __forceinline__ void put_split(uint8_t* hi, uint8_t* lo, int r, int u, const float* v) {
-  uint4 h, l;
-  split2(v[0], v[1], h.x, l.x);
-  split2(v[2], v[3], h.y, l.y);
-  split2(v[4], v[5], h.z, l.z);
-  split2(v[6], v[7], h.w, l.w);
-  put_unit(hi, r, u, h);
-  put_unit(lo, r, u, l);
+// Eight values' parts, a 16-byte unit each.
+__device__ __forceinline__ void split_unit(const float* v, uint4& h, uint4& m, uint4& l) {
+  split3(v[0], v[1], h.x, m.x, l.x);
+  split3(v[2], v[3], h.y, m.y, l.y);
+  split3(v[4], v[5], h.z, m.z, l.z);
+  split3(v[6], v[7], h.w, m.w, l.w);
 }
+
+// e^(s scale - lse) as a power of two, the argument to 2^-24 of its terms: `c` = scale
+// log2 e and `n` = -lse log2 e as sums of two floats.
+struct Exp2 {
+  float ch, cl, nh, nl;
+  __device__ __forceinline__ Exp2(float scale, float lse) {
+    constexpr float kl = 1.92596299e-8f;  // log2 e - float(log2 e)
+    ch = scale * kLog2e;
+    cl = fmaf(scale, kLog2e, -ch) + scale * kl;
+    nh = -lse * kLog2e;
+    nl = -fmaf(lse, kLog2e, nh) - lse * kl;
+  }
+  __device__ __forceinline__ float operator()(float s) const {
+    return ex2(fmaf(s, ch, nh) + fmaf(s, cl, nl));
+  }
+};
 
 // One head tile: NC boxes of 64 columns.
 template <int NC>
@@ -218,10 +240,10 @@ __device__ __noinline__ void restage_dkv(const GenArgs& a, int b, int h, int t0,
 
 // ============================================================ backward: dQ
 // For L > 128: per query tile, Drow, then per key tile S and dP (128 + 128 TMEM
-// columns), dS = P (dP - Drow) scale as hi + lo (hi over the consumed V), the
-// product dS K into the S columns, accumulated in registers.  112 KB (NC = 1:
-// two CTAs per SM) or 160 KB.
-template <int NC> constexpr int dq_smem() { return 3 * NC * (int)kChunk + 2 * (int)kP; }
+// columns), dS = P (dP - Drow) scale as three parts (the first over the consumed V),
+// the product dS K into the S columns, accumulated in registers.  NC = 1: 112 KB, two
+// CTAs per SM, the third part through the first's buffer; NC = 2: 192 KB.
+template <int NC> constexpr int dq_smem() { return 3 * NC * (int)kChunk + (NC + 1) * (int)kP; }
 
 template <int NC>
 __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
@@ -236,8 +258,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
   uint8_t* sdO = smem + kT;
   uint8_t* sK = smem + 2 * kT;
   uint8_t* sV = smem + 3 * kT;
-  uint8_t* sSh = sV;        // dS hi over V (and, NC = 1, the 16 KB after it)
-  uint8_t* sSl = sV + kP;   // dS lo
+  uint8_t* sS = sV;  // dS's parts, kP apart, over V (and, NC = 1, the 16 KB after it)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dq_smem<NC>());  // loads, S/dP, dQ
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 3);
 
@@ -282,8 +303,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
   const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
   const int nk = (a.x.dh + 15) / 16;
   if (row_ok && hf == 0) a.Drow[lrow] = drow;
-  const float nl2 = row_ok ? -a.x.lse[lrow] * kLog2e : 0.f;
-  const float sl2 = a.x.scale * kLog2e, ndr = -drow * a.x.scale;
+  const Exp2 prob(a.x.scale, row_ok ? a.x.lse[lrow] : 0.f);
   float acc[OC];
 #pragma unroll
   for (int c = 0; c < OC; ++c) acc[c] = 0.f;
@@ -306,6 +326,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
     __syncwarp();
     ok = tc::mbar_wait(&bar[1], kt & 1, a.status) && ok;
     tc::fence_after_sync();
+    uint4 last[8];  // NC = 1: the third parts
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int k0 = hf * 64 + c * 32;
@@ -317,29 +338,51 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const bool vis = use && row_ok && (!diag || k0 + j <= r);
-        s[j] = vis ? ex2(fmaf(s[j], sl2, nl2)) * fmaf(dp[j], a.x.scale, ndr) : 0.f;
+        s[j] = vis ? prob(s[j]) * (dp[j] - drow) * a.x.scale : 0.f;
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) put_split(sSh, sSl, r, hf * 8 + c * 4 + u, s + 8 * u);
+      for (int u = 0; u < 4; ++u) {
+        uint4 hm[2];
+        split_unit(s + 8 * u, hm[0], hm[1], last[4 * c + u]);
+        put_unit(sS, r, hf * 8 + c * 4 + u, hm[0]);
+        put_unit(sS + kP, r, hf * 8 + c * 4 + u, hm[1]);
+        if (NC == 2) put_unit(sS + 2 * kP, r, hf * 8 + c * 4 + u, last[4 * c + u]);
+      }
     }
     tc::fence_proxy_async_smem();
     tc::fence_before_sync();
     __syncthreads();  // dS is in place, S and dP are read
+    const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
+    const int nkk = diag ? (tt.rows + 15) / 16 : 8;
     if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
-      if (ok) {
-        const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
-        const int nkk = diag ? (tt.rows + 15) / 16 : 8;
-        for (int kk = 0; kk < nkk; ++kk) {
-          tc::mma_bf16(tmem, p_kmaj(sSh, 0, kk), d_mnmaj(sK, kk), idQ, kk > 0 ? 1u : 0u);
-          tc::mma_bf16(tmem, p_kmaj(sSl, 0, kk), d_mnmaj(sK, kk), idQ, 1u);
-        }
-      }
+      if (ok)
+        for (int part = NC; part >= 0; --part)  // the smallest first
+          for (int kk = 0; kk < nkk; ++kk)
+            tc::mma_bf16(tmem, p_kmaj(sS + part * kP, 0, kk), d_mnmaj(sK, kk), idQ,
+                         part < NC || kk > 0 ? 1u : 0u);
       tc::mma_commit(&bar[2]);
     }
     __syncwarp();
-    ok = tc::mbar_wait(&bar[2], kt & 1, a.status) && ok;
+    ok = tc::mbar_wait(&bar[2], NC == 1 ? 0u : (uint32_t)(kt & 1), a.status) && ok;
     tc::fence_after_sync();
+    if (NC == 1) {  // the third part, in the first's place
+#pragma unroll
+      for (int u = 0; u < 8; ++u) put_unit(sS, r, hf * 8 + u, last[u]);
+      tc::fence_proxy_async_smem();
+      tc::fence_before_sync();
+      __syncthreads();
+      if (warp0 && tc::elect_one()) {
+        tc::fence_after_sync();
+        if (ok)
+          for (int kk = 0; kk < nkk; ++kk)
+            tc::mma_bf16(tmem, p_kmaj(sS, 0, kk), d_mnmaj(sK, kk), idQ, 1u);
+        tc::mma_commit(&bar[2]);
+      }
+      __syncwarp();
+      ok = tc::mbar_wait(&bar[2], 1u, a.status) && ok;
+      tc::fence_after_sync();
+    }
     if (warp0 && tc::elect_one() && kt < tt.j) {  // K, V and dS are consumed: the next key tile
       tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
       load_tile<NC>(sK, &mK, &bar[0], h, tt.kstart + (kt + 1) * kTile, b);
@@ -357,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
 
   const unsigned bad = row_ok ? bad_units<OC>(acc, hf * OC, a.x.dh) : 0u;
   stage_half<NC>(sQ, r, hf, acc);
-  if (__syncthreads_or(bad)) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, bad, sSh);
+  if (__syncthreads_or(bad)) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, bad, sS);
   tc::fence_proxy_async_smem();
   __syncthreads();
   if (warp0 && tc::elect_one() && ok) {
@@ -370,15 +413,17 @@ __global__ void __launch_bounds__(kThreads, NC == 1 ? 2 : 1)
 }
 
 // ====================================================== backward: dK, dV (dQ)
-// Per key tile, its query tiles in turn: S = Q K^T and dP = dO V^T, P as
-// hi + lo for dV += P^T dO, dS = P (dP - Drow) scale, which waits in fp32 in
-// dP's TMEM columns until the dV product has consumed P, as hi + lo in P's
-// buffers for dK += dS^T Q.  FUSED (L <= 128: the key tile is its own and only
-// query tile): Drow is computed here and dQ = dS K joins; P hi covers the
-// consumed V (112 / 160 KB), and the products reuse the columns of S and dP
-// (NC = 1: 256 columns, two CTAs per SM).
+// Per key tile, its query tiles in turn: S = Q K^T and dP = dO V^T, P as three parts
+// for dV += P^T dO, dS = P (dP - Drow) scale, which waits in fp32 in dP's TMEM columns
+// until the dV product has consumed P, as three parts in P's buffers for dK += dS^T Q.
+// FUSED (L <= 128: the key tile is its own and only query tile): Drow is computed
+// here and dQ = dS K joins; P's first part covers the consumed V, and the products
+// reuse the columns of S and dP.  At NC = 1 that form has two buffers (112 KB and 256
+// columns, two CTAs per SM) and three rounds of products: P's first two parts; its
+// third and dS's first; dS's others.
+template <int NC, bool FUSED> constexpr int dkv_parts() { return FUSED && NC == 1 ? 2 : 3; }
 template <int NC, bool FUSED> constexpr int dkv_smem() {
-  return (FUSED ? 3 : 4) * NC * (int)kChunk + 2 * (int)kP;
+  return (FUSED ? 3 : 4) * NC * (int)kChunk + dkv_parts<NC, FUSED>() * (int)kP;
 }
 template <int NC, bool FUSED> constexpr int dkv_cols() { return FUSED && NC == 1 ? 256 : 512; }
 
@@ -392,13 +437,13 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t kT = NC * kChunk;
   constexpr int OC = 32 * NC;
+  constexpr int PARTS = dkv_parts<NC, FUSED>();
   constexpr uint32_t kDV = FUSED ? 0 : 256, kDK = kDV + 64 * NC, kDQ = FUSED ? 128 * NC : 0;
   uint8_t* sQ = smem;              // Q; FUSED: then dQ staging
   uint8_t* sdO = smem + kT;        // dO; then dV staging
   uint8_t* sK = smem + 2 * kT;     // K; then dK staging
   uint8_t* sV = smem + 3 * kT;
-  uint8_t* sPh = FUSED ? sV : smem + 4 * kT;  // P hi, then dS hi
-  uint8_t* sPl = sPh + kP;                    // P lo, then dS lo
+  uint8_t* sP = FUSED ? sV : smem + 4 * kT;  // the parts of P, then of dS, kP apart
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + dkv_smem<NC, FUSED>());  // loads, S/dP, dV, dK
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 4);
 
@@ -446,18 +491,35 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   const uint32_t idMN = tc::idesc_bf16(128, nk * 16, 1, 1);
   const int rbs = FUSED ? (r / a.x.L) * a.x.L : 0;
   const int wbs = FUSED ? ((q * 32) / a.x.L) * a.x.L : 0;
-  const float sl2 = a.x.scale * kLog2e;
   bool ok = true;
 
+  // products over the query rows with one part: dst (+)= part^T t, dQ (+)= part K
+  // (operand descriptors formed once; a step along one adds its bytes / 16)
+  const uint64_t pT = tc::sdesc(tc::smem_u32(sP), kChunk, 1024),
+                 pK = tc::sdesc(tc::smem_u32(sP), 16, 1024), bQ = d_mnmaj(sQ, 0),
+                 bO = d_mnmaj(sdO, 0), bK = d_mnmaj(sK, 0);
+  auto times_t = [&](uint32_t dst, int part, uint64_t t, int nkk, bool first) {
+    const uint64_t p = pT + part * (kP / 16);
+#pragma unroll 4
+    for (int kk = 0; kk < nkk; ++kk)
+      tc::mma_bf16(tmem + dst, p + kk * 128, t + kk * 128, idMN, first && kk == 0 ? 0u : 1u);
+  };
+  auto times_k = [&](int part, int nkk, bool first) {
+    const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
+    const uint64_t p = pK + part * (kP / 16);
+#pragma unroll 4
+    for (int kk = 0; kk < nkk; ++kk)
+      tc::mma_bf16(tmem + kDQ, p + (kk >> 2) * 1024 + (kk & 3) * 2, bK + kk * 128, idQ,
+                   first && kk == 0 ? 0u : 1u);
+  };
   for (int i = tt.j, it = 0; i < jend; ++i, ++it) {  // FUSED: j = 0, jend = 1
     const bool diag = it == 0;
     const int t0 = FUSED ? tt.t0 : tt.kstart + i * kTile;
     const int rows = FUSED ? tt.rows : min(min(kTile, a.x.L - i * kTile), a.x.T - t0);
     const bool row_ok = r < rows;
     const long lrow = ((long)b * a.x.H + h) * a.x.T + t0 + r;
-    const float nl2 = row_ok ? -a.x.lse[lrow] * kLog2e : 0.f;
+    const Exp2 prob(a.x.scale, row_ok ? a.x.lse[lrow] : 0.f);
     if (!FUSED) drow = row_ok ? a.Drow[lrow] : 0.f;
-    const float ndr = -drow * a.x.scale;
     if (warp0 && tc::elect_one()) {
       const bool okk = tc::mbar_wait(&bar[0], it & 1, a.status);
       tc::fence_after_sync();
@@ -474,6 +536,7 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     ok = tc::mbar_wait(&bar[1], it & 1, a.status) && ok;
     tc::fence_after_sync();
     // P to shared memory, dS (fp32) over dP in TMEM
+    uint4 third[8];  // two buffers: P's third parts, then dS's second and third
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int k0 = hf * 64 + c * 32;
@@ -486,12 +549,19 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
       for (int j = 0; j < 32; ++j) {
         const int kk = k0 + j;
         const bool vis = use && row_ok && (!diag || (kk >= rbs && kk <= r));
-        s[j] = vis ? ex2(fmaf(s[j], sl2, nl2)) : 0.f;
-        dp[j] = vis ? s[j] * fmaf(dp[j], a.x.scale, ndr) : 0.f;
+        s[j] = vis ? prob(s[j]) : 0.f;
+        dp[j] = vis ? s[j] * (dp[j] - drow) * a.x.scale : 0.f;
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) put_split(sPh, sPl, r, hf * 8 + c * 4 + u, s + 8 * u);
       tc::tmem_st32(trow + 128u + (uint32_t)k0, dp);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int unit = hf * 8 + c * 4 + u;
+        uint4 h, m;
+        split_unit(s + 8 * u, h, m, third[4 * c + u]);
+        put_unit(sP, r, unit, h);
+        put_unit(sP + kP, r, unit, m);
+        if (PARTS == 3) put_unit(sP + 2 * kP, r, unit, third[4 * c + u]);
+      }
     }
     tc::tmem_st_wait();
     tc::fence_proxy_async_smem();
@@ -500,24 +570,33 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     const int nkk = (rows + 15) / 16;  // queries past the tile's rows have P = dS = 0
     if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
-      if (ok) {
-        for (int kk = 0; kk < nkk; ++kk) {  // dV += P^T dO
-          tc::mma_bf16(tmem + kDV, d_mnmaj(sPh, kk), d_mnmaj(sdO, kk), idMN,
-                       (it > 0 || kk > 0) ? 1u : 0u);
-          tc::mma_bf16(tmem + kDV, d_mnmaj(sPl, kk), d_mnmaj(sdO, kk), idMN, 1u);
-        }
-      }
+      if (ok)
+        for (int part = PARTS - 1; part >= 0; --part)  // dV += P^T dO, the smallest first
+          times_t(kDV, part, bO, nkk, it == 0 && part == PARTS - 1);
       tc::mma_commit(&bar[2]);
     }
     __syncwarp();
     ok = tc::mbar_wait(&bar[2], it & 1, a.status) && ok;
     tc::fence_after_sync();
+    uint4 second[8];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       float ds[32];
       tc::tmem_ld32(trow + 128u + (uint32_t)(hf * 64 + c * 32), ds);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) put_split(sPh, sPl, r, hf * 8 + c * 4 + u, ds + 8 * u);
+      for (int u = 0; u < 4; ++u) {
+        const int unit = hf * 8 + c * 4 + u;
+        if (PARTS == 2) put_unit(sP, r, unit, third[4 * c + u]);
+        uint4 h;
+        split_unit(ds + 8 * u, h, second[4 * c + u], third[4 * c + u]);
+        if (PARTS == 2) {
+          put_unit(sP + kP, r, unit, h);
+        } else {
+          put_unit(sP, r, unit, h);
+          put_unit(sP + kP, r, unit, second[4 * c + u]);
+          put_unit(sP + 2 * kP, r, unit, third[4 * c + u]);
+        }
+      }
     }
     tc::fence_proxy_async_smem();
     tc::fence_before_sync();
@@ -525,17 +604,15 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     if (warp0 && tc::elect_one()) {
       tc::fence_after_sync();
       if (ok) {
-        for (int kk = 0; kk < nkk; ++kk) {  // dK += dS^T Q
-          tc::mma_bf16(tmem + kDK, d_mnmaj(sPh, kk), d_mnmaj(sQ, kk), idMN,
-                       (it > 0 || kk > 0) ? 1u : 0u);
-          tc::mma_bf16(tmem + kDK, d_mnmaj(sPl, kk), d_mnmaj(sQ, kk), idMN, 1u);
-        }
-        if (FUSED) {
-          const uint32_t idQ = tc::idesc_bf16(128, nk * 16, 0, 1);
-          for (int kk = 0; kk < nkk; ++kk) {  // dQ = dS K
-            tc::mma_bf16(tmem + kDQ, p_kmaj(sPh, 0, kk), d_mnmaj(sK, kk), idQ, kk > 0 ? 1u : 0u);
-            tc::mma_bf16(tmem + kDQ, p_kmaj(sPl, 0, kk), d_mnmaj(sK, kk), idQ, 1u);
-          }
+        if (PARTS == 2) {
+          times_t(kDV, 0, bO, nkk, false);
+          times_t(kDK, 1, bQ, nkk, true);
+          times_k(1, nkk, true);
+        } else {
+          for (int part = 2; part >= 0; --part)  // dK += dS^T Q, dQ = dS K
+            times_t(kDK, part, bQ, nkk, it == 0 && part == 2);
+          if (FUSED)
+            for (int part = 2; part >= 0; --part) times_k(part, nkk, part == 2);
         }
       }
       tc::mma_commit(&bar[3]);
@@ -543,6 +620,28 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
     __syncwarp();
     ok = tc::mbar_wait(&bar[3], it & 1, a.status) && ok;
     tc::fence_after_sync();
+    if (PARTS == 2) {  // dS's other parts
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        put_unit(sP, r, hf * 8 + u, second[u]);
+        put_unit(sP + kP, r, hf * 8 + u, third[u]);
+      }
+      tc::fence_proxy_async_smem();
+      tc::fence_before_sync();
+      __syncthreads();
+      if (warp0 && tc::elect_one()) {
+        tc::fence_after_sync();
+        if (ok)
+          for (int part = 0; part < 2; ++part) {
+            times_t(kDK, part, bQ, nkk, false);
+            times_k(part, nkk, false);
+          }
+        tc::mma_commit(&bar[3]);
+      }
+      __syncwarp();
+      ok = tc::mbar_wait(&bar[3], 1u, a.status) && ok;
+      tc::fence_after_sync();
+    }
     if (!FUSED && warp0 && tc::elect_one() && i + 1 < jend) {  // the next query tile
       tc::mbar_arrive_expect_tx(&bar[0], 2 * kT);
       load_tile<NC>(sQ, &mQ, &bar[0], h, t0 + kTile, b);
@@ -561,9 +660,9 @@ __global__ void __launch_bounds__(kThreads, FUSED && NC == 1 ? 2 : 1)
   const unsigned badv = staged(kDV, sdO), badk = staged(kDK, sK),
                  badq = FUSED ? staged(kDQ, sQ) : 0u;
   if (__syncthreads_or(badk | badv | badq)) {
-    restage_dkv(a, b, h, tt.t0, sK, sdO, r, hf * OC / 8, badk, badv, sPh);
+    restage_dkv(a, b, h, tt.t0, sK, sdO, r, hf * OC / 8, badk, badv, sP);
     __syncthreads();
-    if (FUSED) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, badq, sPh);
+    if (FUSED) restage_dq(a, b, h, tt.t0, sQ, r, hf * OC / 8, badq, sP);
   }
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
