@@ -85,6 +85,8 @@ def _load():
     lib.bcmt_test_set_tensor_cores.restype = ctypes.c_int
     lib.bcmt_test_set_side_streams.argtypes = [ctypes.c_int]
     lib.bcmt_test_set_side_streams.restype = None
+    lib.bcmt_test_set_decode_one_launch.argtypes = [ctypes.c_int]
+    lib.bcmt_test_set_decode_one_launch.restype = None
     lib.bcmt_test_gemm.argtypes = [ctypes.c_int] * 6 + [_VP, ctypes.c_long, ctypes.c_long, _VP,
                                                         ctypes.c_long, ctypes.c_long, _VP,
                                                         ctypes.c_long, ctypes.c_int, _VP]
@@ -108,7 +110,8 @@ EXPORTED = ("bcmt_workspace_size", "bcmt_scratch_size", "bcmt_forward", "bcmt_ba
             "bcmt_device_status", "bcmt_last_error", "bcmt_profile_read", "bcmt_profile_reset",
             "bcmt_attention_backward_noalloc",
             "bcmt_decode_state_size", "bcmt_decode_reset", "bcmt_decode_step",
-            "bcmt_test_set_tensor_cores", "bcmt_test_set_side_streams", "bcmt_test_gemm", "bcmt_test_gemm_group", "bcmt_test_attn",
+            "bcmt_test_set_tensor_cores", "bcmt_test_set_side_streams",
+            "bcmt_test_set_decode_one_launch", "bcmt_test_gemm", "bcmt_test_gemm_group", "bcmt_test_attn",
             "bcmt_test_wait_expiry")
 
 
@@ -232,6 +235,10 @@ def bcmt_test_set_tensor_cores(gemm_on: bool, attn_on: bool) -> int:
 
 def bcmt_test_set_side_streams(on: bool) -> None:
     LIB.bcmt_test_set_side_streams(int(on))
+
+
+def bcmt_test_set_decode_one_launch(on: bool) -> None:
+    LIB.bcmt_test_set_decode_one_launch(int(on))
 
 
 def bcmt_test_gemm(impl, dtype, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, splits=1,

@@ -974,11 +974,13 @@ cudaError_t step_cluster(const Launch& lc, const DecodeArgs& a) {
 }
 }  // namespace
 
+bool g_decode_one_launch = true;  // switchable only through bcmt_testing.h
+
 // bf16: one launch (step_cluster) where the shape fits it; fp32 (whose products
 // are fp32 multiply-adds) and the rest: a launch per stage.
 cudaError_t decode_step(const Launch& lc, int dtype, const DecodeArgs& a) {
   if (a.L > kMaxL || a.dh > 128) return cudaErrorInvalidValue;
-  if (dtype == 1) {
+  if (dtype == 1 && g_decode_one_launch) {
     const cudaError_t e = step_cluster<1>(lc, a);
     if (e != cudaErrorNotSupported) return e;
   }

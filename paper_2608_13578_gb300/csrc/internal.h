@@ -283,5 +283,6 @@ struct DecodeArgs {
   DecodeState s;
 };
 cudaError_t decode_step(const Launch& lc, int dtype, const DecodeArgs& a);
+extern bool g_decode_one_launch;  // false: every step as a launch per stage
 
 }  // namespace bcmt

@@ -50,3 +50,24 @@ def test_one_pass_backward(C, B, T, H, dh, L, pad):
         assert np.isfinite(x).all(), n
         assert np.abs(x - r).max() <= 2e-2 * max(np.abs(r).max(), top), n
         assert np.abs(x - y.double().cpu().numpy()).max() <= 2 ** -6 * top, n
+
+
+@pytest.mark.parametrize("B,T,H,dh,L", [(1, 700, 2, 64, 256), (2, 600, 4, 16, 512), (1, 400, 2, 32, 384)])
+@pytest.mark.parametrize("which,value", [("v", float("inf")), ("dO", float("nan")), ("k", float("nan")),
+                                         ("q", float("inf"))])
+def test_non_finite_tokens(C, B, T, H, dh, L, which, value):
+    """A non-finite token reaches the rows that see it (where the CUDA-core kernels have
+    it), nothing that it does not reach in the two-kernel form (hidden rows of its tile),
+    and no other head, block or sequence: those are the same bit for bit."""
+    ins = dict(zip(("q", "k", "v", "dO"), (t.cuda() for t in _inputs(B, T, H, dh))))
+    D = H * dh
+    p = C.make_params(B, T, D, H, L, "bf16")
+    clean = _run(C, 4, p, B, T, D, H, *ins.values())[2]
+    ins[which][0, 130, 5] = value
+    blk, two, simt = (_run(C, impl, p, B, T, D, H, *ins.values())[2] for impl in (4, 2, 0))
+    for x, y, s, z in zip(blk, two, simt, clean):
+        assert not (torch.isfinite(x) & ~torch.isfinite(s)).any()
+        assert not (~torch.isfinite(x) & torch.isfinite(y)).any()
+        assert torch.equal(x[..., dh:], z[..., dh:]) and torch.equal(x[1:], z[1:])
+        assert torch.equal(x[:, L:], z[:, L:])
+    assert any(not torch.isfinite(x).all() for x in blk)
