@@ -22,6 +22,8 @@
 // L64 fp32 forward 516 and 48 us, backward 2002 and 92 us; B4 T2048 D1024 h8 L128
 // bf16 forward 1997 and 126 us; B4 T1000 D768 h8 L48 bf16 forward 306 and 63 us.
 // Deterministic: every sum runs in a fixed order.
+#include <limits.h>
+
 #include <algorithm>
 
 #include "attn_slow.cuh"
@@ -744,7 +746,8 @@ SimtArgs<E> simt_args(const AttnArgs& f, const AttnBwdArgs* ab) {
   a.lse = f.lse;
   a.Drow = ab ? ab->Drow : nullptr;
   a.rows = f.L <= kTile ? (kTile / f.L) * f.L : kTile;
-  a.tpb = f.L <= kTile ? 1 : (f.L + kTile - 1) / kTile;
+  // (a block is no longer than the sequence: no tiles for the rest of it)
+  a.tpb = f.L <= kTile ? 1 : (std::min(f.L, f.T) + kTile - 1) / kTile;
   a.nb = f.L <= kTile ? (f.T + a.rows - 1) / a.rows : (f.T + f.L - 1) / f.L;
   a.B = f.B;
   // rows of q, k, v and of the gradients may have any stride; those of O and dO
@@ -767,7 +770,9 @@ cudaError_t simt_launch(const Launch& lc, K kern, std::atomic<unsigned long long
   if (cudaError_t e = smem_opt_in(kern, simt_smem(std::max(tiles, 3), max_cols, kMaxDh), opted);
       e != cudaSuccess)
     return e;
-  cudaError_t e = launch_k(kern, dim3((unsigned)a.nb * a.tpb * f.H * f.B), dim3(kThreads),
+  const double grid = (double)a.nb * a.tpb * f.H * f.B;
+  if (grid > INT_MAX) return cudaErrorInvalidConfiguration;
+  cudaError_t e = launch_k(kern, dim3((unsigned)grid), dim3(kThreads),
                            simt_smem(tiles, cols, f.dh), lc.stream, a, x...);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
