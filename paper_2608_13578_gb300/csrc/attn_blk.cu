@@ -228,7 +228,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::tma_load_3d(sK + (c & 1) * G::tile, &mK, &bar_k[c & 1], i.h * DH, i.t0 + kt * kTile, i.b);
         tc::tma_load_3d(sV + (c & 1) * G::tile, &mV, &bar_k[c & 1], i.h * DH, i.t0 + kt * kTile, i.b);
       };
+      uint32_t qn = 0, qodd = 0;  // slots loaded so far, and those an odd number of times
       auto load_q = [&](const Item& i, int qt) {
+        qn |= 1u << qt;
+        qodd ^= 1u << qt;
         tc::mbar_arrive_expect_tx(&bar_q[qt], 2 * G::tile);
         tc::tma_load_3d(sQ + qt * G::tile, &mQ, &bar_q[qt], i.h * DH, i.t0 + qt * kTile, i.b);
         tc::tma_load_3d(sdO + qt * G::tile, &mdO, &bar_q[qt], i.h * DH, i.t0 + qt * kTile, i.b);
@@ -268,6 +271,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
+      if (!ok) {  // a wait has run out: what is on its way has to land before the CTA ends
+        for (int qt = 0; qt < kMaxM; ++qt)
+          if (qn >> qt & 1u) tc::mbar_wait(&bar_q[qt], (qodd >> qt & 1u) ^ 1u, a.status);
+        for (int n = max(kc - 2, 0); n < kc; ++n)
+          tc::mbar_wait(&bar_k[n & 1], (n >> 1) & 1, a.status);
+      }
     }
     __syncwarp();
   } else if (warp >= kStatWarp) {
@@ -282,11 +291,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       return t;
     };
     // its O on the way to shared memory and its log-sum-exp into v
+    int loads = 0;  // of O, by the lane that issues them
     auto fetch = [&](At t, float* v) {
       if (t.it >= a.total) return;
       const Item j(a, t.it);
       const int r0 = j.t0 + t.qt * kTile;
       if (warp == kStatWarp && tc::elect_one() && ok) {
+        ++loads;
         tc::mbar_arrive_expect_tx(bar_o, G::tile);
         tc::tma_load_3d(sO, &mO, bar_o, j.h * DH, r0, j.b);
       }
@@ -333,6 +344,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       t = after(t);
       fetch(t, ls);
     }
+    if (!ok && loads > 0) tc::mbar_wait(bar_o, (loads - 1) & 1, a.status);  // as the loads above
+    __syncwarp();
   } else {
     // ------------------------------------------------- elementwise, results
     const int q = warp & 3, hf = warp >> 2;
