@@ -263,9 +263,6 @@ int sm_count() {
   return n;
 }
 
-namespace {
-}  // namespace
-
 // Persistent, warp-specialised tcgen05 GEMM.  Tiles are 128 x BN output
 // blocks (optionally one K-split each), taken round-robin by the CTAs, m
 // fastest.  Warp 0 / lane 0 streams 64-deep K slices of A and B into a

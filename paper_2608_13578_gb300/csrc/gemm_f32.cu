@@ -482,17 +482,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ========================================================================= host
 namespace {
-int sms() {
-  static int n = 0;
-  if (!n) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 1;
-  }
-  return n;
-}
-
 template <int BN, bool A_MN, bool B_MN, class Epi>
 cudaError_t launch(const Launch& lc, int M, int N, int K, const Operand& A, const Operand& B,
                    const Epi& epi, const EpiArgs& ea, int splits) {
@@ -510,7 +499,7 @@ cudaError_t launch(const Launch& lc, int M, int N, int K, const Operand& A, cons
     return cudaErrorInvalidValue;
   const int nkb = (K + kBK - 1) / kBK, kps = (nkb + splits - 1) / splits;
   const int tm = (M + kBM - 1) / kBM, tn = (N + BN - 1) / BN, tiles = tm * tn * splits;
-  cudaError_t e = launch_k(kern, dim3(tiles < sms() ? tiles : sms()), dim3(kThreads), C::SMEM,
+  cudaError_t e = launch_k(kern, dim3(tiles < sm_count() ? tiles : sm_count()), dim3(kThreads), C::SMEM,
                            lc.stream, A, B, mC, M, N, K, kps, tm, tn, tiles, epi, lc.status);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -559,7 +548,7 @@ cudaError_t gemm_f32(const Launch& lc, int M, int N, int K, const void* A, long 
   splits = (epi == EPI_PARTIAL) ? effective_splits(K, splits) : 1;
   // 64-wide tiles spread a product that would leave half of the SMs idle
   const long tiles = (long)((M + kBM - 1) / kBM) * ((N + 127) / 128) * splits;
-  if (tiles * 2 <= sms()) return pick_layout<64>(lc, M, N, K, a, b, epi, ea, splits);
+  if (tiles * 2 <= sm_count()) return pick_layout<64>(lc, M, N, K, a, b, epi, ea, splits);
   return pick_layout<128>(lc, M, N, K, a, b, epi, ea, splits);
 }
 

@@ -12,6 +12,7 @@ struct Launch {
   cudaStream_t stream;
   unsigned* status;  // device status word (bounded waits OR bits into it)
 };
+int sm_count();  // SMs of the current device (of the first one asked about)
 
 // ----------------------------------------------------------------- GEMM
 // C[M,N] = A[M,K] B[K,N] with fp32 accumulation, element (m,k) of A at
@@ -195,7 +196,6 @@ bool attn_tc_supported(int dtype, int dh, int L);
 bool attn_fl_supported(int dtype, int dh, int L);
 cudaError_t attn_fwd_fl(const Launch& lc, const AttnArgs& a);
 cudaError_t attn_bwd_fl(const Launch& lc, const AttnBwdArgs& a);
-int sm_count();  // SMs of the current device (of the first one asked about)
 
 // The backward of blocks of several tiles in one pass (also writes Drow), where its
 // accumulators fit TMEM.
