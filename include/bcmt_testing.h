@@ -29,10 +29,10 @@ int bcmt_test_set_tensor_cores(int gemm_on, int attn_on);
  * default): the side streams are used. */
 void bcmt_test_set_side_streams(int on);
 
-/* on = 0: bcmt_decode_step runs bf16 tokens as a launch per stage from now on in this
- * process, as it does sizes that the one-launch step does not hold; 1 (the default): in
- * one launch where they fit.  Switch only between sequences (bcmt_decode_reset). */
-void bcmt_test_set_decode_one_launch(int on);
+/* How bcmt_decode_step runs bf16 tokens from now on in this process: mode 0 as a launch
+ * per stage, 1 (the default) in one launch where that fits and is the faster form, 2 in
+ * one launch wherever it fits.  Switch only between sequences (bcmt_decode_reset). */
+void bcmt_test_set_decode_one_launch(int mode);
 
 /* C[M,N] = A[M,K] B[K,N] with fp32 accumulation, element (m,k) of A at
  * A[m*sam + k*sak] and (k,n) of B at B[k*sbk + n*sbn] (elements, not bytes);

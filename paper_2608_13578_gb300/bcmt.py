@@ -237,8 +237,8 @@ def bcmt_test_set_side_streams(on: bool) -> None:
     LIB.bcmt_test_set_side_streams(int(on))
 
 
-def bcmt_test_set_decode_one_launch(on: bool) -> None:
-    LIB.bcmt_test_set_decode_one_launch(int(on))
+def bcmt_test_set_decode_one_launch(mode: int) -> None:
+    LIB.bcmt_test_set_decode_one_launch(int(mode))
 
 
 def bcmt_test_gemm(impl, dtype, dtype_out, M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, splits=1,

@@ -1240,7 +1240,7 @@ int bcmt_test_set_tensor_cores(int gemm_on, int attn_on) {
 
 void bcmt_test_set_side_streams(int on) { g_use_side_streams = on != 0; }
 
-void bcmt_test_set_decode_one_launch(int on) { g_decode_one_launch = on != 0; }
+void bcmt_test_set_decode_one_launch(int mode) { g_decode_one_launch = mode; }
 
 int bcmt_test_wait_expiry(long long cycles, void* stream) {
   if (cycles < 1 || cycles > tc::kWaitCycles) {

@@ -13,8 +13,8 @@
 // Values the full forward stores in the storage dtype (Q/K/V, Concat(heads),
 // H, M) are rounded to it here too, so that a decoded token reproduces the
 // forward's output row.  bf16 steps run as one launch (decode_cluster_kernel);
-// fp32 steps, and bf16 shapes too large for it, as a launch per stage, whose
-// vector-matrix products stream each weight once on CUDA cores.
+// fp32 steps, and bf16 shapes too large for it or faster so (staged_is_faster), as a
+// launch per stage, whose vector-matrix products stream each weight once on CUDA cores.
 #include <algorithm>
 
 #include "common.cuh"
@@ -22,6 +22,8 @@
 #include "tc.cuh"
 
 namespace bcmt {
+
+int g_decode_one_launch = 1;  // switchable only through bcmt_testing.h
 
 namespace {
 constexpr int kMaxL = 1024;
@@ -908,12 +910,29 @@ DecodeFit decode_fit() {
   return {(v - 1) / 64, (v - 1) % 64};
 }
 
+// Sizes that fit one launch and are faster as a launch per stage, which has all SMs at
+// work (us a token, staged and one launch, in the last quarter of a block):
+//   one sequence of a wide layer, whose weights one cluster's SMs have to bring alone:
+//     D = 1280 27 and 37 (L 16), 31 and 37 (L 64), 46 and 42 (L 256); 2048 43 and 51, 47 and
+//     51, 63 and 56; from two sequences on the other way round (D = 1280 41 and 37, L 16);
+//   many sequences of a narrow layer, sixteen to a cluster: B = 64, D = 64 23 and 24 (L 16),
+//     44 and 40 (L 256); D = 256 24 and 27, 46 and 43; at B = 48 24 and 23 (D = 256, L 16), at
+//     D = 384 37 and 28;
+//   more sequences than the clusters that run at a time hold (seven, 112 sequences):
+//     B = 128, D = 128 24 and 50 (L 16), D = 512 52 and 57, D = 640 100 and 66.
+bool staged_is_faster(const DecodeArgs& a, int clusters) {
+  if (a.B == 1) return a.D > 1024 && a.L < 256;
+  if (a.B > kDecRows * clusters) return a.D < 640;
+  return a.B > 48 && a.D < 384 && a.L < 256;
+}
+
 // The whole step in one launch; cudaErrorNotSupported for shapes whose rows do
-// not fit a CTA's shared memory.
+// not fit a CTA's shared memory, and for those above.
 template <int NT>
 cudaError_t step_cluster(const Launch& lc, const DecodeArgs& a) {
   const DecodeFit fit = decode_fit<NT>();
   if (!fit.ctas) return cudaErrorNotSupported;
+  if (g_decode_one_launch == 1 && staged_is_faster(a, fit.clusters)) return cudaErrorNotSupported;
   // sequences per cluster: over up to kDecClusters clusters, at most kDecRows each
   int ncl = std::min(a.B, std::min(fit.clusters, kDecClusters));
   if (a.B > ncl * kDecRows) ncl = (a.B + kDecRows - 1) / kDecRows;
@@ -974,13 +993,11 @@ cudaError_t step_cluster(const Launch& lc, const DecodeArgs& a) {
 }
 }  // namespace
 
-bool g_decode_one_launch = true;  // switchable only through bcmt_testing.h
-
 // bf16: one launch (step_cluster) where the shape fits it; fp32 (whose products
 // are fp32 multiply-adds) and the rest: a launch per stage.
 cudaError_t decode_step(const Launch& lc, int dtype, const DecodeArgs& a) {
   if (a.L > kMaxL || a.dh > 128) return cudaErrorInvalidValue;
-  if (dtype == 1 && g_decode_one_launch) {
+  if (dtype == 1 && g_decode_one_launch != 0) {
     const cudaError_t e = step_cluster<1>(lc, a);
     if (e != cudaErrorNotSupported) return e;
   }

@@ -283,6 +283,7 @@ struct DecodeArgs {
   DecodeState s;
 };
 cudaError_t decode_step(const Launch& lc, int dtype, const DecodeArgs& a);
-extern bool g_decode_one_launch;  // false: every step as a launch per stage
+// bf16 steps in one launch: 0 never, 1 where that is the faster form, 2 wherever it fits
+extern int g_decode_one_launch;
 
 }  // namespace bcmt
